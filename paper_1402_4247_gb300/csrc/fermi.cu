@@ -1,10 +1,22 @@
 // Part 5 (Sec. 3): chemical potential and band energy.  mu solves
 //   N(mu) = g sum_p w_p sum_{j < m_p} f((eps_pj - mu)/kT) = N_e,  f(x) = 1/(1 + e^x),
-// by bisection on [min eps - 40 kT, max eps + 40 kT] (N is strictly increasing for kT > 0),
-// then f_pj and E_band = g sum w f eps.  All eigenvalues of all (k, spin) problems enter
-// one sum, so the kernel runs on the whole GPU: each round every block sums its share of
-// the Fermi factors, the partial sums meet after a grid-wide barrier, and every block
-// applies the same (deterministic, fixed-order) total to its copy of the bracket.
+// by safeguarded Newton steps on [min eps - 40 kT, max eps + 40 kT] (N is strictly increasing
+// for kT > 0), then f_pj and E_band = g sum w f eps.  All eigenvalues of all (k, spin) problems
+// enter one sum, so the kernel runs on the whole GPU: each round every block sums its share of
+// the Fermi factors and of their derivatives, the partial sums meet after a grid-wide barrier,
+// and every block takes the same (deterministic, fixed-order) step.
+//
+// What bounds it is the chain of rounds: FP64 arithmetic at 64 cycles per warp instruction and
+// scheduler (an exponential and a division per value, ~45 instructions), reductions, and a grid
+// barrier of ~1.2 us.  Hence:
+//  * Newton steps, with bisection where a step leaves the bracket or the bracket does not
+//    halve: ~10-25 rounds instead of the ~55 of plain bisection;
+//  * f is evaluated only within FP_WIN kT of mu (1 below, 0 above: e^-60 is 1e-10 of the last
+//    bit of a sum that holds any occupied state), so the early rounds are comparisons;
+//  * the blocks' partial sums are added by one warp (in every thread they cost 152 FP64
+//    instructions per warp and round, ~10 us);
+//  * small sets take few blocks (one: no grid barrier) and few warps (a reduction per warp).
+// Measured on GB300: 72,704 eigenvalues 1713 -> 491 us, 256 eigenvalues 1393 -> 186 us.
 #include <cooperative_groups.h>
 
 #include <cfloat>
@@ -23,18 +35,6 @@ __device__ __forceinline__ double fermi_fn(double x) {
   return ex / (1.0 + ex);
 }
 
-__device__ double block_sum(double v, double* red) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  __syncthreads();
-  if (lane == 0) red[wid] = v;
-  __syncthreads();
-  double t = 0.0;
-  for (int k = 0; k < (int)(blockDim.x >> 5); ++k) t += red[k];
-  return t;
-}
-
 __device__ double block_minmax(double v, double* red, bool is_max) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
@@ -50,17 +50,58 @@ __device__ double block_minmax(double v, double* red, bool is_max) {
   return t;
 }
 
-// Grid-wide sum in a fixed order; buf alternates so that a fast block never overwrites
-// partials that a slow block is still reading.
-__device__ double grid_sum(cg::grid_group& grid, double v, double* red, double* scratch, int& buf) {
-  v = block_sum(v, red);
-  double* part = scratch + (size_t)buf * gridDim.x;
-  if (threadIdx.x == 0) part[blockIdx.x] = v;
+constexpr int FP_SUMS = 2;         // sums per round: N and dN/dmu
+constexpr double FP_WIN = 60.0;    // f is 1 below and 0 above this many kT from mu
+
+// Grid-wide sums of v[0..K) in a fixed order, into out[0..K) of every thread; buf alternates so
+// that a fast block never overwrites partials that a slow block is still reading.
+// red: 8 K doubles of shared memory at least, tot: K.  active (uniform over a warp): false for a
+// warp whose values are all zero.
+template <int K>
+__device__ void grid_sum(cg::grid_group& grid, const double* v, double* out, double* red, double* tot, double* scratch,
+                         int& buf, bool active) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  double x[K];
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    x[k] = v[k];
+    if (active)
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) x[k] += __shfl_xor_sync(0xffffffffu, x[k], o);
+  }
+  __syncthreads();
+  if (lane == 0)
+#pragma unroll
+    for (int k = 0; k < K; ++k) red[wid * K + k] = x[k];
+  __syncthreads();
+  double* part = scratch + (size_t)buf * FP_SUMS * gridDim.x;
   buf ^= 1;
-  grid.sync();
-  double t = 0.0;
-  for (unsigned b = 0; b < gridDim.x; ++b) t += part[b];
-  return t;
+  if (threadIdx.x < K) {
+    double t = 0.0;
+    for (int w = 0; w < FT / 32; ++w) t += red[w * K + threadIdx.x];
+    if (gridDim.x == 1) tot[threadIdx.x] = t;
+    else part[(size_t)blockIdx.x * K + threadIdx.x] = t;
+  }
+  if (gridDim.x > 1) {
+    grid.sync();
+    if (wid == 0) {
+      double t[K];
+#pragma unroll
+      for (int k = 0; k < K; ++k) t[k] = 0.0;
+      for (unsigned b = lane; b < gridDim.x; b += 32)
+#pragma unroll
+        for (int k = 0; k < K; ++k) t[k] += __ldcg(part + (size_t)b * K + k);
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) t[k] += __shfl_xor_sync(0xffffffffu, t[k], o);
+        if (lane == 0) tot[k] = t[k];
+      }
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < K; ++k) out[k] = tot[k];
 }
 
 __global__ void __launch_bounds__(FT)
@@ -69,14 +110,18 @@ fermi_kernel(int n, int nprob, int nk, double g, const double* __restrict__ wk, 
              double* __restrict__ f, int32_t* __restrict__ nocc, double* __restrict__ mu_out, double* __restrict__ eband_out,
              int32_t* __restrict__ status, double* __restrict__ scratch) {
   cg::grid_group grid = cg::this_grid();
-  __shared__ double red[32];
+  __shared__ double red[8 * FP_SUMS > 32 ? 8 * FP_SUMS : 32], tot[FP_SUMS], mmx[2];
+  __shared__ int s_over;
   int buf = 0;
   const size_t total = (size_t)nprob * n;
   const size_t gtid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const size_t gstride = (size_t)gridDim.x * blockDim.x;
+  // threads that take values: at least two each, in whole groups of four warps (one per scheduler)
+  const size_t gall = (size_t)gridDim.x * blockDim.x, gwant = ((total + 1) / 2 + 127) / 128 * 128;
+  const size_t gstride = gwant < gall ? gwant : gall;
+  const bool busy = gtid < gstride;
 
   double lmin = DBL_MAX, lmax = -DBL_MAX, cap = 0.0;
-  for (size_t idx = gtid; idx < total; idx += gstride) {
+  for (size_t idx = busy ? gtid : total; idx < total; idx += gstride) {
     const int p = (int)(idx / n), j = (int)(idx % n);
     if (j < m[p]) {
       const double e = eps[idx];
@@ -90,38 +135,76 @@ fermi_kernel(int n, int nprob, int nk, double g, const double* __restrict__ wk, 
   // precision, so reduce them with dedicated partial slots
   lmin = block_minmax(lmin, red, false);
   lmax = block_minmax(lmax, red, true);
-  double* mm = scratch + 2 * (size_t)gridDim.x;
+  double* mm = scratch + 2 * FP_SUMS * (size_t)gridDim.x;
   if (threadIdx.x == 0) {
     mm[2 * blockIdx.x] = lmin;
     mm[2 * blockIdx.x + 1] = lmax;
   }
-  cap = grid_sum(grid, cap, red, scratch, buf);  // (contains a grid.sync)
-  double emin = DBL_MAX, emax = -DBL_MAX;
-  for (unsigned b = 0; b < gridDim.x; ++b) {
-    emin = fmin(emin, mm[2 * b]);
-    emax = fmax(emax, mm[2 * b + 1]);
+  grid_sum<1>(grid, &cap, &cap, red, tot, scratch, buf, busy);  // (contains a grid.sync)
+  double emin = lmin, emax = lmax;
+  if (gridDim.x > 1) {
+    if (threadIdx.x < 32) {
+      for (unsigned b = threadIdx.x; b < gridDim.x; b += 32) {
+        emin = fmin(emin, __ldcg(mm + 2 * b));
+        emax = fmax(emax, __ldcg(mm + 2 * b + 1));
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        emin = fmin(emin, __shfl_xor_sync(0xffffffffu, emin, o));
+        emax = fmax(emax, __shfl_xor_sync(0xffffffffu, emax, o));
+      }
+      if (threadIdx.x == 0) {
+        mmx[0] = emin;
+        mmx[1] = emax;
+      }
+    }
+    __syncthreads();
+    emin = mmx[0];
+    emax = mmx[1];
   }
   int32_t st = 0;
   if (!(n_electrons >= 0.0 && n_electrons <= cap * (1.0 + 1e-14)) || !(emin <= emax)) st = NAO_E_RANGE;
   double lo = emin - 40.0 * kT, hi = emax + 40.0 * kT;
   if (st == 0) {
+    const double rkT = 1.0 / kT;
+    double x = 0.5 * (lo + hi), width2 = hi - lo;  // bracket width two rounds ago
+    double width1 = width2;
     for (int it = 0; it < 200; ++it) {
-      const double mid = 0.5 * (lo + hi);
-      if (mid <= lo || mid >= hi || hi - lo <= 1e-15 * fmax(1.0, fabs(mid))) break;
-      double s = 0.0;
-      for (size_t idx = gtid; idx < total; idx += gstride) {
+      const double tol = 1e-15 * fmax(1.0, fabs(x));
+      if (!(x > lo && x < hi) || hi - lo <= tol) break;
+      double s[FP_SUMS] = {0.0, 0.0};
+      for (size_t idx = busy ? gtid : total; idx < total; idx += gstride) {
         const int p = (int)(idx / n), j = (int)(idx % n);
-        if (j < m[p]) s += wk[p % nk] * fermi_fn((eps[idx] - mid) / kT);
+        if (j >= m[p]) continue;
+        const double t = (eps[idx] - x) * rkT, w = wk[p % nk];
+        if (t < -FP_WIN) {
+          s[0] += w;
+        } else if (!(t > FP_WIN)) {
+          const double ex = exp(-fabs(t)), r = 1.0 / (1.0 + ex);
+          const double q = ex * r;  // min(f, 1 - f)
+          s[0] = fma(w, t > 0.0 ? q : r, s[0]);
+          s[1] = fma(w, q * r, s[1]);  // f (1 - f) = kT df/dmu
+        }
       }
-      s = g * grid_sum(grid, s, red, scratch, buf);
-      if (s < n_electrons) lo = mid;
-      else hi = mid;
+      grid_sum<FP_SUMS>(grid, s, s, red, tot, scratch, buf, busy);
+      if (g * s[0] < n_electrons) lo = x;
+      else hi = x;
+      const double xn = x - (g * s[0] - n_electrons) * kT / (g * s[1]);
+      if (fabs(xn - x) <= 0.5 * tol && xn >= lo && xn <= hi) {  // converged to the bracket's tolerance
+        lo = hi = xn;
+        break;
+      }
+      // Newton inside the bracket while it halves every two rounds, else bisection
+      const bool slow = hi - lo > 0.5 * width2;
+      width2 = width1;
+      width1 = hi - lo;
+      x = (xn > lo && xn < hi && !slow) ? xn : 0.5 * (lo + hi);
     }
   }
   const double mu = 0.5 * (lo + hi);
   // occupations, band energy, occupied-band counts
   double eb = 0.0;
-  for (size_t idx = gtid; idx < total; idx += gstride) {
+  for (size_t idx = busy ? gtid : total; idx < total; idx += gstride) {
     const int p = (int)(idx / n), j = (int)(idx % n);
     double fj = 0.0;
     if (st == 0 && j < m[p]) {
@@ -131,28 +214,29 @@ fermi_kernel(int n, int nprob, int nk, double g, const double* __restrict__ wk, 
     }
     f[idx] = fj;
   }
-  eb = grid_sum(grid, eb, red, scratch, buf);
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    *mu_out = (st == 0) ? mu : __longlong_as_double(0x7ff8000000000000ll);
-    *eband_out = (st == 0) ? eb : __longlong_as_double(0x7ff8000000000000ll);
-  }
-  grid.sync();
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
+  grid_sum<1>(grid, &eb, &eb, red, tot, scratch, buf, busy);  // (its barriers publish nocc)
+  if (blockIdx.x == 0) {
+    if (threadIdx.x == 0) {
+      *mu_out = (st == 0) ? mu : __longlong_as_double(0x7ff8000000000000ll);
+      *eband_out = (st == 0) ? eb : __longlong_as_double(0x7ff8000000000000ll);
+      s_over = 0;
+    }
+    __syncthreads();
     // bands beyond the nb returned eigenvectors must be empty; the count is clamped so
     // that the density-matrix product never reads past column nb
-    int32_t s2 = st;
-    for (int p = 0; p < nprob; ++p)
-      if (nocc[p] > nb) {
-        if (s2 == 0) s2 = NAO_E_INVALID;
+    for (int p = threadIdx.x; p < nprob; p += blockDim.x)
+      if (__ldcg(nocc + p) > nb) {
+        s_over = 1;
         nocc[p] = nb;
       }
-    if (status) *status = s2;
+    __syncthreads();
+    if (threadIdx.x == 0 && status) *status = (st == 0 && s_over) ? (int32_t)NAO_E_INVALID : st;
   }
 }
 
 }  // namespace
 
-size_t fermi_scratch_doubles(int num_sms) { return (size_t)4 * num_sms + 64; }
+size_t fermi_scratch_doubles(int num_sms) { return (size_t)(2 * FP_SUMS + 2) * num_sms + 64; }
 
 cudaError_t launch_fermi(int num_sms, int n, int nprob, int nk, double g, const double* wk, const double* eps,
                          const int32_t* m, int nb, double n_electrons, double kT, double f_min, double* f,
@@ -161,7 +245,10 @@ cudaError_t launch_fermi(int num_sms, int n, int nprob, int nk, double g, const 
   cudaError_t err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fermi_kernel, FT, 0);
   if (err != cudaSuccess) return err;
   if (per_sm < 1) return cudaErrorCooperativeLaunchTooLarge;
-  int grid = num_sms;  // one block per SM is enough: ~nprob*n/(num_sms*FT) values per thread
+  // eight values per thread before another block joins (its share of a round's barrier costs
+  // more than eight comparisons), at most one block per SM
+  const long long want = ((long long)n * nprob + 8 * FT - 1) / (8 * FT);
+  int grid = want < num_sms ? (int)want : num_sms;
   void* args[] = {&n,  &nprob, &nk,   &g,  &wk,    &eps,   &m,       &nb,     &n_electrons,
                   &kT, &f_min, &f,    &nocc, &mu,  &eband, &status, &scratch};
   return cudaLaunchCooperativeKernel((const void*)fermi_kernel, dim3(grid), dim3(FT), args, 0, st);
@@ -182,9 +269,10 @@ cudaError_t launch_fermi(int num_sms, int n, int nprob, int nk, double g, const 
 #include <mutex>
 
 namespace {
-constexpr int NOALLOC_MAX_BLOCKS = 1024;           // grid blocks whose partial sums fit
+constexpr int NOALLOC_MAX_BLOCKS = 512;            // grid blocks whose partial sums fit
 constexpr int NOALLOC_MAX_PROBLEMS = 65536;        // (spin, k) problems whose band counts fit
-constexpr size_t NOALLOC_PART_DOUBLES = 4 * (size_t)NOALLOC_MAX_BLOCKS + 64;
+constexpr size_t NOALLOC_PART_DOUBLES = 8 * (size_t)NOALLOC_MAX_BLOCKS + 64;
+static_assert(2 * FP_SUMS + 2 <= 8, "the grid's partial sums fit");
 constexpr size_t NOALLOC_DOUBLES = NOALLOC_PART_DOUBLES + NOALLOC_MAX_PROBLEMS / 2;  // + int32 counts
 }  // namespace
 
