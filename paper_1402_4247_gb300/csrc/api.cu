@@ -308,7 +308,9 @@ cudaError_t backtransform_blocked(nao_ctx* ctx, int n, int nprob, const int32_t*
                                   const z64* tau, const double* Z, const double* w, int use_rsqrt, z64* U, z64* Vf,
                                   z64* tauc, z64* G, z64* T, z64* W, z64* VT, void* ozws, cudaStream_t st,
                                   int digits, int lowest, int off = 1, const Q2Ref* q2 = nullptr) {
-  const int nb = NAO_WY_NB;
+  // blocks of 128 reflectors; up to 64 reflectors take one block of 64 (T's FP64 work falls
+  // eightfold, and nothing has to be joined)
+  const int nb = n - off <= NAO_WY_T ? NAO_WY_T : NAO_WY_NB;
   const int ncolv = (n + nb - 1) / nb * nb;
   const long long snn = (long long)n * n, svf = (long long)n * ncolv, snb2 = (long long)nb * nb,
                   snbn = (long long)nb * n;
@@ -337,6 +339,17 @@ cudaError_t backtransform_blocked(nao_ctx* ctx, int n, int nprob, const int32_t*
   if (nblk > 0) {
     NaoStage stage_(ctx, "backtransform", st, 1);
     e = launch_build_t(nb, nprob, nblk, G, tauc, ncolv, T, st);
+    if (e != cudaSuccess) return e;
+  }
+  if (nblk > 0 && nb > NAO_WY_T) {
+    // the halves of every T_j joined: T12 = -T11 (G12 T22), as batches of all blocks and problems
+    constexpr int h = NAO_WY_T;
+    const GemmDims dj{h, h, h, nullptr, nullptr, nullptr, 0};
+    e = run_zgemm(ctx, "backtransform", nprob * nblk, dj, 1.0, GemmOperand{G + h, snb2, nb, 1, 0, nullptr},
+                  GemmOperand{T + (size_t)h * nb + h, snb2, nb, 1, 0, nullptr}, 0.0, W, (long long)h * h, h, 1, ozws, st);
+    if (e != cudaSuccess) return e;
+    e = run_zgemm(ctx, "backtransform", nprob * nblk, dj, -1.0, GemmOperand{T, snb2, nb, 1, 0, nullptr},
+                  GemmOperand{W, (long long)h * h, h, 1, 0, nullptr}, 0.0, T + h, snb2, nb, 1, ozws, st);
     if (e != cudaSuccess) return e;
   }
   for (int j = 0; j < nblk; ++j) {  // VT_j = V_j T_j (rows x nb; T_j upper triangular, row-major)

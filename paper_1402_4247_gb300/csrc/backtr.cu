@@ -164,57 +164,94 @@ __global__ void init_u_kernel(int n, const int32_t* __restrict__ size, const int
 }
 
 // T (nb x nb, row-major, upper triangular) of block j from G = V^H V (row-major, Hermitian):
-// T_ii = tau_i, T(0:i, i) = -tau_i T(0:i, 0:i) G(0:i, i).  One block of nb threads per
-// (block j, problem p); thread r owns row r of T, which it writes and reads back itself (in
-// global memory, cached).  Columns are formed BT_B at a time: the part of each dot product
-// over the finished columns is accumulated for all BT_B new columns from one read of the row
-// (the reads of T fall BT_B-fold), then the new columns follow one by one from registers;
-// the terms are added in the same order as one column at a time.  G's columns of the batch
-// sit in shared memory (row stride BT_B + 1: no bank conflicts).  G and T of block j of
-// problem p at (j nprob + p) nb^2.
-constexpr int BT_B = 8;
-__global__ void build_t_kernel(int nb, int nprob, const z64* __restrict__ Gbase, const z64* __restrict__ taucbase,
-                               int ncolv, z64* __restrict__ Tbase) {
-  extern __shared__ z64 gs[];  // G(c, i0 + k) at gs[c (BT_B + 1) + k]
-  const int p = blockIdx.x % nprob, j = blockIdx.x / nprob;
-  const int r = threadIdx.x;
-  const z64* G = Gbase + (size_t)blockIdx.x * nb * nb;
-  const z64* tau = taucbase + (size_t)p * ncolv + (size_t)j * nb;
-  z64* Tr = Tbase + (size_t)blockIdx.x * nb * nb + (size_t)r * nb;  // row r
-  for (int c = 0; c < r; ++c) Tr[c] = zmk(0.0, 0.0);
-  for (int i0 = 0; i0 < nb; i0 += BT_B) {
-    const int nbat = nb - i0 < BT_B ? nb - i0 : BT_B, L = i0 + nbat;
-    __syncthreads();  // the previous batch's reads of gs are done
-    // G(c, i) = conj(G(i, c)) (G is Hermitian): coalesced loads of rows i0 .. i0 + nbat - 1
-    for (int idx = r; idx < L * nbat; idx += nb) {
-      const int k = idx / L, c = idx - k * L;
-      gs[c * (BT_B + 1) + k] = zconj(G[(size_t)(i0 + k) * nb + c]);
+// T_ii = tau_i, T(0:i, i) = -tau_i T(0:i, 0:i) G(0:i, i).  One block of 256 threads forms the
+// diagonal BT_H x BT_H part of T (of sub-block blockIdx.x % nsub) in shared memory, by halves:
+//   T = [T11 T12; 0 T22] with T12 = -T11 (G12 T22),
+// from 16 x 16 diagonal blocks formed by the column recurrence (a warp each, two lanes per
+// row) through 16 -> 32 -> 64; the caller joins the two halves of a 128-column block with
+// two tensor-core products.  FP64 bounds it (64^3/6 complex multiply-adds, 40 us of one SM's
+// FP64 pipe, with every lane busy; one thread per row over the whole block, the form before, was a
+// chain of 128^2/2 multiply-adds).  Back-transformation stage per step, before -> now: n = 64, 4
+// problems 2.82 -> 0.49 ms; n = 129, 12 problems 2.87 -> 0.77 ms; n = 568, 128 problems 39.8 -> 36.8 ms.
+// G and T of block j of problem p at (j nprob + p) nb^2.
+constexpr int BT_H = NAO_WY_T;
+constexpr int BT_THREADS = 256;
+constexpr int BT_LD = BT_H + 1;
+
+// X = G12 T22, then T12 = -T11 X for the pairs of h x h blocks along the diagonal
+template <int H>
+__device__ __forceinline__ void bt_join(const z64* __restrict__ g, z64* __restrict__ t, z64* __restrict__ x) {
+  constexpr int NP = BT_H / (2 * H), TOT = NP * H * H;
+  static_assert(TOT % BT_THREADS == 0, "whole passes");
+#pragma unroll
+  for (int o = 0; o < TOT / BT_THREADS; ++o) {  // lanes along the rows: one c (and k range) per warp
+    const int idx = threadIdx.x + o * BT_THREADS;
+    const int pr = idx / (H * H), r = idx % H, c = (idx / H) % H, b = pr * 2 * H;
+    z64 acc = zmk(0.0, 0.0);
+    for (int k = 0; k <= c; ++k) acc = zfma(g[(b + r) * BT_LD + b + H + k], t[(b + H + k) * BT_LD + b + H + c], acc);
+    x[(pr * H + r) * (H + 1) + c] = acc;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int o = 0; o < TOT / BT_THREADS; ++o) {  // lanes along the columns: one r (and k range) per warp
+    const int idx = threadIdx.x + o * BT_THREADS;
+    const int pr = idx / (H * H), c = idx % H, r = (idx / H) % H, b = pr * 2 * H;
+    z64 acc = zmk(0.0, 0.0);
+    for (int k = r; k < H; ++k) acc = zfma(t[(b + r) * BT_LD + b + k], x[(pr * H + k) * (H + 1) + c], acc);
+    t[(b + r) * BT_LD + b + H + c] = zmk(-acc.x, -acc.y);
+  }
+  __syncthreads();
+}
+
+__global__ void __launch_bounds__(BT_THREADS)
+build_t_kernel(int nb, int nprob, int nsub, const z64* __restrict__ Gbase, const z64* __restrict__ taucbase,
+               int ncolv, z64* __restrict__ Tbase) {
+  extern __shared__ z64 bts[];
+  z64* g = bts;                       // [BT_H][BT_LD]
+  z64* t = g + BT_H * BT_LD;          // [BT_H][BT_LD]
+  z64* x = t + BT_H * BT_LD;          // [BT_H / 2][BT_H / 2 + 1]
+  const int q = blockIdx.x / nsub, p = q % nprob, j = q / nprob;
+  const int s0 = blockIdx.x % nsub * BT_H, H = nb - s0 < BT_H ? nb - s0 : BT_H;  // this sub-block's columns
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const z64* G = Gbase + (size_t)q * nb * nb + (size_t)s0 * nb + s0;
+  const z64* tau = taucbase + (size_t)p * ncolv + (size_t)j * nb + s0;
+  z64* T = Tbase + (size_t)q * nb * nb;
+  // rows s0 .. of T outside the diagonal sub-block: zero (the join writes the upper ones)
+  for (int idx = tid; idx < H * nb; idx += BT_THREADS) {
+    const int r = idx / nb, c = idx % nb;
+    if (c < s0 || c >= s0 + H) T[(size_t)(s0 + r) * nb + c] = zmk(0.0, 0.0);
+  }
+  bool any = false;
+  if (tid < H) any = tau[tid].x != 0.0 || tau[tid].y != 0.0;
+  if (!__syncthreads_or(any)) {  // no reflector here: T = 0
+    for (int idx = tid; idx < H * H; idx += BT_THREADS)
+      T[(size_t)(s0 + idx / H) * nb + s0 + idx % H] = zmk(0.0, 0.0);
+    return;
+  }
+  for (int idx = tid; idx < BT_H * BT_H; idx += BT_THREADS) {
+    const int r = idx / BT_H, c = idx % BT_H;
+    g[r * BT_LD + c] = (r < H && c < H) ? G[(size_t)r * nb + c] : zmk(0.0, 0.0);
+    t[r * BT_LD + c] = zmk(0.0, 0.0);
+  }
+  __syncthreads();
+  if (wid < BT_H / 16) {  // T(r, i) = -tau_i sum_{r <= c < i} T(r, c) G(c, i) on the diagonal blocks
+    const int b = 16 * wid, r = lane & 15, h = lane >> 4;
+    for (int i = 0; i < 16; ++i) {
+      const z64 ti = b + i < H ? tau[b + i] : zmk(0.0, 0.0);
+      z64 acc = zmk(0.0, 0.0);
+      for (int c = h; c < i; c += 2) acc = zfma(t[(b + r) * BT_LD + b + c], g[(b + c) * BT_LD + b + i], acc);
+      acc.x += __shfl_xor_sync(0xffffffffu, acc.x, 16);
+      acc.y += __shfl_xor_sync(0xffffffffu, acc.y, 16);
+      if (h == 0 && r <= i) t[(b + r) * BT_LD + b + i] = r == i ? ti : zmul(zmk(-ti.x, -ti.y), acc);
+      __syncwarp();
     }
-    __syncthreads();
-    z64 acc[BT_B], tb[BT_B];
-#pragma unroll
-    for (int k = 0; k < BT_B; ++k) acc[k] = zmk(0.0, 0.0);
-    for (int c = r; c < i0; ++c) {  // finished columns
-      const z64 t = Tr[c];
-#pragma unroll
-      for (int k = 0; k < BT_B; ++k) acc[k] = zfma(t, gs[c * (BT_B + 1) + k], acc[k]);
-    }
-#pragma unroll
-    for (int k = 0; k < BT_B; ++k) {
-      if (k < nbat) {
-        const int i = i0 + k;
-        z64 a = acc[k];
-#pragma unroll
-        for (int c2 = 0; c2 < k; ++c2)  // the batch's earlier columns c = i0 + c2 >= r
-          if (i0 + c2 >= r) a = zfma(tb[c2], gs[(i0 + c2) * (BT_B + 1) + k], a);
-        const z64 ti = tau[i];
-        z64 tv = zmk(0.0, 0.0);
-        if (r < i) tv = zmul(zmk(-ti.x, -ti.y), a);
-        else if (r == i) tv = ti;
-        tb[k] = tv;
-        if (r <= i) Tr[i] = tv;
-      }
-    }
+  }
+  __syncthreads();
+  bt_join<16>(g, t, x);
+  if (BT_H > 32) bt_join<32>(g, t, x);
+  for (int idx = tid; idx < H * H; idx += BT_THREADS) {
+    const int r = idx / H, c = idx % H;
+    T[(size_t)(s0 + r) * nb + s0 + c] = t[r * BT_LD + c];
   }
 }
 
@@ -256,8 +293,11 @@ cudaError_t launch_init_u(int n, int nprob, const int32_t* size, const int32_t* 
 
 cudaError_t launch_build_t(int nb, int nprob, int nblk, const z64* G, const z64* tauc, int ncolv, z64* T,
                            cudaStream_t st) {
-  const size_t smem = (size_t)nb * (BT_B + 1) * sizeof(z64);
-  build_t_kernel<<<nprob * nblk, nb, smem, st>>>(nb, nprob, G, tauc, ncolv, T);
+  const size_t smem = (2 * (size_t)BT_H * BT_LD + (size_t)(BT_H / 2) * (BT_H / 2 + 1)) * sizeof(z64);
+  const cudaError_t e = cudaFuncSetAttribute(build_t_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  const int nsub = (nb + BT_H - 1) / BT_H;
+  build_t_kernel<<<nprob * nblk * nsub, BT_THREADS, smem, st>>>(nb, nprob, nsub, G, tauc, ncolv, T);
   return cudaGetLastError();
 }
 

@@ -224,6 +224,7 @@ cudaError_t launch_stein(int n, int nprob, const int32_t* size, const double* d,
 
 // Blocked (compact WY) back-transformation helpers, see backtr.cu.
 constexpr int NAO_WY_NB = 128;
+constexpr int NAO_WY_T = 64;  // T_j is formed in diagonal blocks of this order, joined by products
 // off: row of reflector i's head is i + off (1: one-stage; B: stage 1 of the two-stage form)
 cudaError_t launch_extract_v(int n, int nprob, const int32_t* size, const z64* A, int lda, long long strideA,
                              const z64* tau, long long strideV, int ncolv, z64* V, int ldv, long long strideVf,
@@ -231,7 +232,8 @@ cudaError_t launch_extract_v(int n, int nprob, const int32_t* size, const z64* A
 // init_u: column c of U takes Z's column m - nc + c (the top nc) or, when lowest, column c.
 cudaError_t launch_init_u(int n, int nprob, const int32_t* size, const int32_t* ncols, const double* Z, int ldz,
                           long long strideZ, z64* U, int ldu, long long strideU, int lowest, cudaStream_t st);
-// T_j of every WY block j < nblk and problem p at once: G_j, T_j at (j nprob + p) nb^2.
+// The diagonal blocks of order NAO_WY_T of T_j (zero elsewhere; all of T_j when nb <= NAO_WY_T)
+// for every WY block j < nblk and problem p at once: G_j, T_j at (j nprob + p) nb^2.
 cudaError_t launch_build_t(int nb, int nprob, int nblk, const z64* G, const z64* tauc, int ncolv, z64* T,
                            cudaStream_t st);
 cudaError_t launch_normalize_cols(int n, int nprob, const int32_t* size, const int32_t* ncols, const double* w,
