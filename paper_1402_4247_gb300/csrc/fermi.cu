@@ -10,13 +10,14 @@
 // scheduler (an exponential and a division per value, ~45 instructions), reductions, and a grid
 // barrier of ~1.2 us.  Hence:
 //  * Newton steps, with bisection where a step leaves the bracket or the bracket does not
-//    halve: ~10-25 rounds instead of the ~55 of plain bisection;
+//    halve, and the bracket closed around the root at the end: ~15-30 rounds instead of the
+//    ~55 of plain bisection;
 //  * f is evaluated only within FP_WIN kT of mu (1 below, 0 above: e^-60 is 1e-10 of the last
 //    bit of a sum that holds any occupied state), so the early rounds are comparisons;
 //  * the blocks' partial sums are added by one warp (in every thread they cost 152 FP64
 //    instructions per warp and round, ~10 us);
 //  * small sets take few blocks (one: no grid barrier) and few warps (a reduction per warp).
-// Measured on GB300: 72,704 eigenvalues 1713 -> 491 us, 256 eigenvalues 1393 -> 186 us.
+// Measured on GB300: 72,704 eigenvalues 1713 -> 500 us, 256 eigenvalues 1393 -> 200 us.
 #include <cooperative_groups.h>
 
 #include <cfloat>
@@ -50,7 +51,7 @@ __device__ double block_minmax(double v, double* red, bool is_max) {
   return t;
 }
 
-constexpr int FP_SUMS = 2;         // sums per round: N and dN/dmu
+constexpr int FP_SUMS = 3;         // sums per round: states below mu, their and the others' tails, dN/dmu
 constexpr double FP_WIN = 60.0;    // f is 1 below and 0 above this many kT from mu
 
 // Grid-wide sums of v[0..K) in a fixed order, into out[0..K) of every thread; buf alternates so
@@ -168,37 +169,42 @@ fermi_kernel(int n, int nprob, int nk, double g, const double* __restrict__ wk, 
   if (st == 0) {
     const double rkT = 1.0 / kT;
     double x = 0.5 * (lo + hi), width2 = hi - lo;  // bracket width two rounds ago
-    double width1 = width2;
+    double width1 = width2, reach = 1.0;
     for (int it = 0; it < 200; ++it) {
-      const double tol = 1e-15 * fmax(1.0, fabs(x));
-      if (!(x > lo && x < hi) || hi - lo <= tol) break;
-      double s[FP_SUMS] = {0.0, 0.0};
+      const double mid = 0.5 * (lo + hi), tol = 1e-15 * fmax(1.0, fabs(mid));
+      if (mid <= lo || mid >= hi || hi - lo <= tol) break;
+      // N - N_e = (states below x - N_e) + tails, the tails (f above x, f - 1 below) summed by
+      // themselves: inside a gap N is flat to its rounding, and only their sum places mu
+      double s[FP_SUMS] = {0.0, 0.0, 0.0};
       for (size_t idx = busy ? gtid : total; idx < total; idx += gstride) {
         const int p = (int)(idx / n), j = (int)(idx % n);
         if (j >= m[p]) continue;
         const double t = (eps[idx] - x) * rkT, w = wk[p % nk];
-        if (t < -FP_WIN) {
-          s[0] += w;
-        } else if (!(t > FP_WIN)) {
+        if (!(t > 0.0)) s[0] += w;
+        if (!(fabs(t) > FP_WIN)) {
           const double ex = exp(-fabs(t)), r = 1.0 / (1.0 + ex);
           const double q = ex * r;  // min(f, 1 - f)
-          s[0] = fma(w, t > 0.0 ? q : r, s[0]);
-          s[1] = fma(w, q * r, s[1]);  // f (1 - f) = kT df/dmu
+          s[1] = fma(t > 0.0 ? w : -w, q, s[1]);
+          s[2] = fma(w, q * r, s[2]);  // f (1 - f) = kT df/dmu
         }
       }
       grid_sum<FP_SUMS>(grid, s, s, red, tot, scratch, buf, busy);
-      if (g * s[0] < n_electrons) lo = x;
+      const double excess = fma(g, s[0], -n_electrons) + g * s[1];
+      const bool below = excess < 0.0;
+      if (below) lo = x;
       else hi = x;
-      const double xn = x - (g * s[0] - n_electrons) * kT / (g * s[1]);
-      if (fabs(xn - x) <= 0.5 * tol && xn >= lo && xn <= hi) {  // converged to the bracket's tolerance
-        lo = hi = xn;
-        break;
+      const double step = -excess * kT / (g * s[2]);
+      double xn = x + step;
+      if (!(fabs(step) > 16.0 * tol)) {  // at the root: close the bracket from its other side
+        const double w = fmax(2.0 * fabs(step), tol) * reach;
+        xn = below ? x + w : x - w;
+        reach *= 8.0;
+      } else if (hi - lo > 0.5 * width2) {  // Newton while the bracket halves every two rounds
+        xn = hi;                            // (bisects)
       }
-      // Newton inside the bracket while it halves every two rounds, else bisection
-      const bool slow = hi - lo > 0.5 * width2;
       width2 = width1;
       width1 = hi - lo;
-      x = (xn > lo && xn < hi && !slow) ? xn : 0.5 * (lo + hi);
+      x = (xn > lo && xn < hi) ? xn : 0.5 * (lo + hi);
     }
   }
   const double mu = 0.5 * (lo + hi);
