@@ -180,7 +180,7 @@ cudaError_t run_dgemm(nao_ctx* ctx, const char* stage, int nprob, GemmDims d, do
 
 // Workspace layout of nao_gen_eig (byte offsets into the context's arena) and its size.
 struct GenEigPlan {
-  size_t oAS, oTauS, odS, oeS, owS, oZ, oZ2, oG, oScr, omS, ostS, oX, oHf, oY, oHp, oV, oTauH, odH, oeH, owH, omP, onbP, ostP, ostH, oOz, oVf, oTc, oG2, oT2, oW, oW2, oVW, oDig, oErow;
+  size_t oAS, oTauS, odS, oeS, owS, oZ, oZ2, oG, oScr, omS, ostS, oX, oHf, oY, oHp, oV, oTauH, odH, oeH, owH, omP, onbP, ostP, ostH, oOz, oVf, oTc, oG2, oT2, oW, oW2, oVW, oDig, oErow, oMd;
   // two-stage reduction (band width B2 > 0): V T, the panel's small matrices, band, stage-2 reflectors
   size_t oSVT, oSG, oST, oSM, oSN, oSTc, oSAB, oSV2, oSTau2;
   // split Parts 3-4: the second half's inverse-iteration scratch and product workspace
@@ -239,6 +239,7 @@ GenEigPlan plan_gen_eig(int n, int nprob, int nSe, bool use_tc, int B2, bool spl
   // 8-bit digit planes of the Householder trailing matrix (tensor-core product method)
   W.oDig = P.take<char>(use_tc ? hetrd_digits_bytes(n, nmax, NAO_HT_DIGITS_FP64) : 16);
   W.oErow = P.take<int>((size_t)(n > 1 ? n - 1 : 1) * nmax);
+  W.oMd = P.take<char>(use_tc ? hetrd_panel_bytes(n, nmax) : 16);  // and of its panels
   const size_t b2 = B2 > 0 ? (size_t)B2 : 0;
   const size_t sq = B2 > 0 ? (size_t)sbr_q2_count(n, B2) : 0;
   W.oSVT = P.take<z64>(b2 * n * nmax + 1);
@@ -385,7 +386,7 @@ cudaError_t backtransform_blocked(nao_ctx* ctx, int n, int nprob, const int32_t*
 // (NAO_HT_DIGITS_FP64, or NAO_HT_DIGITS_MIXED for the H' reduction of the mixed mode).
 cudaError_t hetrd_blocked(nao_ctx* ctx, int n, int nprob, const int32_t* size, z64* A, double* d, double* e, z64* tau,
                           z64* VW, void* ozws, cudaStream_t st, int digits, void* dig, int* erow,
-                          int panel_digits = NAO_HT_DIGITS_FP64, int cluster_nprob = 0) {
+                          void* md, int panel_digits = NAO_HT_DIGITS_FP64, int cluster_nprob = 0) {
   // exact integer matrix-vector products with the tensor-core method; FP64 FMAs otherwise
   // (up to the order whose digit words still fit in a block's shared memory)
   const bool use_dig = ctx->gemm_method == NAO_GEMM_TC && dig != nullptr && hetrd_digits_fit(n, panel_digits);
@@ -393,7 +394,8 @@ cudaError_t hetrd_blocked(nao_ctx* ctx, int n, int nprob, const int32_t* size, z
   const int NB = NAO_HT_NB;
   // cluster size from the number of matrices that share the GPU (cluster_nprob: a concurrent
   // launch's matrices included)
-  const int cl = hetrd_cluster_size(n, cluster_nprob > 0 ? cluster_nprob : nprob, ctx->num_sms, pd);
+  const int np = cluster_nprob > 0 ? cluster_nprob : nprob;
+  const int cl = use_dig ? hetrd_mma_cluster_size(n, np, ctx->num_sms, pd) : hetrd_cluster_size(n, np, ctx->num_sms);
   const long long snn = (long long)n * n, svw = (long long)n * 3 * NB;
   for (int i0 = 0; i0 < n; i0 += NB) {
     cudaError_t err = cudaSuccess;
@@ -403,8 +405,11 @@ cudaError_t hetrd_blocked(nao_ctx* ctx, int n, int nprob, const int32_t* size, z
     }
     if (err == cudaSuccess) {
       NaoStage stage_(ctx, "hetrd", st, 1);
-      err = launch_hetrd_panel(n, nprob, size, A, n, snn, d, e, tau, n, VW, svw, i0, cl, use_dig ? dig : nullptr,
-                               erow, pd, VW + (size_t)nprob * svw, st);
+      z64* VWr = VW + (size_t)nprob * svw;
+      if (use_dig)
+        err = launch_hetrd_panel_mma(n, nprob, size, A, n, snn, d, e, tau, n, i0, cl, dig, erow, pd, md, VWr, svw, st);
+      else
+        err = launch_hetrd_panel(n, nprob, size, A, n, snn, d, e, tau, n, VW, svw, i0, cl, VWr, st);
     }
     if (err != cudaSuccess) return err;
     const int r0 = i0 + NB;
@@ -832,6 +837,7 @@ int nao_gen_eig_sized(nao_ctx* ctx, int n, int nprob, const nao_c128* H, const n
   z64 *Vf = (z64*)(ws + W.oVf), *tauc = (z64*)(ws + W.oTc), *Gw = (z64*)(ws + W.oG2), *Tw = (z64*)(ws + W.oT2),
       *Ww = (z64*)(ws + W.oW), *VTw = (z64*)(ws + W.oW2), *VWp = (z64*)(ws + W.oVW);
   void* digp = use_tc ? (void*)(ws + W.oDig) : nullptr;
+  void* mdp = ws + W.oMd;
   int* erowp = (int*)(ws + W.oErow);
   const SbrWork sbr{VWp, (z64*)(ws + W.oSVT), (z64*)(ws + W.oSG), (z64*)(ws + W.oST), (z64*)(ws + W.oSM),
                     (z64*)(ws + W.oSN), (z64*)(ws + W.oSTc), (z64*)(ws + W.oSAB), (z64*)(ws + W.oSV2),
@@ -856,7 +862,7 @@ int nao_gen_eig_sized(nao_ctx* ctx, int n, int nprob, const nao_c128* H, const n
   if (B2 > 0)
     NAO_CUDA_TRY(ctx, hetrd_two_stage(ctx, n, nSe, s_size, AS, dS, eS, tauS, sbr, B2, ozws, st, NAO_OZ_DIGITS_FP64));
   else
-    NAO_CUDA_TRY(ctx, hetrd_blocked(ctx, n, nSe, s_size, AS, dS, eS, tauS, VWp, ozws, st, NAO_OZ_DIGITS_FP64, digp, erowp));
+    NAO_CUDA_TRY(ctx, hetrd_blocked(ctx, n, nSe, s_size, AS, dS, eS, tauS, VWp, ozws, st, NAO_OZ_DIGITS_FP64, digp, erowp, mdp));
   const int mrrr_s = ctx->cfg.mrrr_all ? 2 : ctx->cfg.overlap_mrrr, mrrr_h = ctx->cfg.mrrr_all ? 2 : 0;
   NAO_STAGE("stein", mrrr_s ? 5 : 4,
             launch_stein(n, nSe, s_size, dS, eS, n, wS, Z, n, snn, scr, stS, nullptr, n,
@@ -893,7 +899,7 @@ int nao_gen_eig_sized(nao_ctx* ctx, int n, int nprob, const nao_c128* H, const n
       z64 *Hf, *Y, *Hp, *V, *tauH, *Vf, *tauc, *Gw, *Tw, *Ww, *VTw, *VWp, *C;
       double *dH, *eH, *wH, *Z, *Z2, *G, *scr, *eps;
       int32_t *mP, *nbP, *stH, *nc2;
-      void *ozws, *digp;
+      void *ozws, *digp, *mdp;
       int *erowp, *ns2;
     };
     auto hp_half = [&](int np, cudaStream_t st, const HpHalf& h, cudaEvent_t part3_done) -> int {
@@ -909,7 +915,7 @@ int nao_gen_eig_sized(nao_ctx* ctx, int n, int nprob, const nao_c128* H, const n
       NAO_STAGE("misc", 1, launch_hermitize(n, np, h.mP, h.Hp, n, snn, st));
       if (part3_done) NAO_CUDA_TRY(ctx, cudaEventRecord(part3_done, st));
       NAO_CUDA_TRY(ctx, hetrd_blocked(ctx, n, np, h.mP, h.Hp, h.dH, h.eH, h.tauH, h.VWp, h.ozws, st, dig, h.digp,
-                                      h.erowp, NAO_HT_DIGITS_FP64, nprob));
+                                      h.erowp, h.mdp, NAO_HT_DIGITS_FP64, nprob));
       const int nv_max = C ? n : 0;
       NAO_STAGE("stein", mrrr_h ? 5 : 4, launch_stein(n, np, h.mP, h.dH, h.eH, n, h.wH, h.Z, n, snn, h.scr, h.stH,
                                                      h.nbP, nv_max, ctx->cfg.inverse_iteration_max, mrrr_h, st,
@@ -973,6 +979,7 @@ int nao_gen_eig_sized(nao_ctx* ctx, int n, int nprob, const nao_c128* H, const n
       h.stH = stH + p0;
       h.ozws = oz_h;
       h.digp = dig_h;
+      h.mdp = p0 ? (char*)mdp + hetrd_panel_bytes(n, p0) : (char*)mdp;
       h.erowp = erowp + (size_t)p0 * (n > 1 ? n - 1 : 1);
       h.ns2 = ns2f + p0;
       h.nc2 = nc2 + p0;
@@ -1009,7 +1016,7 @@ int nao_gen_eig_sized(nao_ctx* ctx, int n, int nprob, const nao_c128* H, const n
   if (B2 > 0)
     NAO_CUDA_TRY(ctx, hetrd_two_stage(ctx, n, nprob, mP, Hp, dH, eH, tauH, sbr, B2, ozws, st, dig));
   else
-    NAO_CUDA_TRY(ctx, hetrd_blocked(ctx, n, nprob, mP, Hp, dH, eH, tauH, VWp, ozws, st, dig, digp, erowp,
+    NAO_CUDA_TRY(ctx, hetrd_blocked(ctx, n, nprob, mP, Hp, dH, eH, tauH, VWp, ozws, st, dig, digp, erowp, mdp,
                                     mixed ? NAO_HT_DIGITS_MIXED : NAO_HT_DIGITS_FP64));
   // Eigenvectors of H' only where they are used (the paper's second pass, dstevx's index
   // range): the lowest nb per problem for C, all m for the mixed-mode refinement, none when

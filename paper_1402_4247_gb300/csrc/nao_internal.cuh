@@ -162,25 +162,31 @@ cudaError_t launch_herm_fill(int n, int nprob, const z64* src, long long src_str
 
 // Eigen_HH step 1: Householder tridiagonalization, one block per problem, in place on the
 // full Hermitian column-major matrix A (ld).  size[p] (or n when size == null) is the order.
-// Only the lower triangle of A is read and updated.  `cluster` blocks (1..8, a thread-block
-// cluster) share each matrix; hetrd_cluster_size picks it from the problem count.
-// One launch reduces the panel of columns i0 .. i0+NAO_HT_NB-1; VW ([nprob][3 NB][n], the
-// columns [V | W | V]) receives the panel's reflectors and update vectors, and the caller
-// applies A(i0+NB:, i0+NB:) -= V W^H + W V^H before the next panel.
+// Only the lower triangle of A is read and updated.  `cluster` blocks (a thread-block cluster)
+// share each matrix; the *_cluster_size functions pick it from the problem count.
+// One launch reduces the panel of columns i0 .. i0+NAO_HT_NB-1; VWr ([nprob][n][3 NB], after VW)
+// receives the panel's reflectors and update vectors as rows [V | W | V], and the caller
+// applies A(i0+NB:, i0+NB:) -= V W^H + W V^H before the next panel.  VW: [nprob][3 NB][n] scratch.
 constexpr int NAO_HT_NB = 32;
-// Digit counts of the panel's integer matrix-vector products: 8 (62 bits, FP64 accuracy) or
-// 6 (46 bits: the H' reduction of the mixed mode); 0 selects the FP64 FMA path.
+// Digit counts of the panel's exact matrix-vector products: 8 (62 bits, FP64 accuracy) or
+// 6 (46 bits: the H' reduction of the mixed mode); 0 selects the FP64 form.
 constexpr int NAO_HT_DIGITS_FP64 = 8;
 constexpr int NAO_HT_DIGITS_MIXED = 6;
-int hetrd_cluster_size(int n, int nprob, int num_sms, int digits);
-bool hetrd_digits_fit(int n, int digits);  // the digit path's shared memory fits a block at order n
-// dig / erow (nullable): 8-bit digit planes of the trailing matrix made by launch_hetrd_digits
-// for this panel (with the same digit count); with them the panel forms its Hermitian
-// matrix-vector products exactly with integer dot products (DP4A) instead of FP64 FMAs.
+// FP64 form (csrc/hetrd.cu)
+int hetrd_cluster_size(int n, int nprob, int num_sms);
 cudaError_t launch_hetrd_panel(int n, int nprob, const int32_t* size, z64* A, int ld, long long strideA, double* d,
                                double* e, z64* tau, long long strideV, z64* VW, long long strideVW, int i0, int cluster,
-                               const void* dig, const int* erow, int digits, z64* VWr, cudaStream_t st);
-// digit planes (row exponents: (n - 1) nprob ints)
+                               z64* VWr, cudaStream_t st);
+// digit form (csrc/hetrd_mma.cu).  dig / erow: 8-bit digit tiles of the trailing matrix and the
+// rows' exponents, made by launch_hetrd_digits for this panel with the same digit count
+bool hetrd_digits_fit(int n, int digits);  // its shared memory fits a block at order n
+int hetrd_mma_cluster_size(int n, int nprob, int num_sms, int digits);
+cudaError_t launch_hetrd_panel_mma(int n, int nprob, const int32_t* size, z64* A, int ld, long long strideA, double* d,
+                                   double* e, z64* tau, long long strideV, int i0, int C, const void* dig,
+                                   const int* erow, int digits, void* md, z64* VWr, long long strideVW, cudaStream_t st);
+// md: scratch for the panel's own digits (hetrd_panel_bytes)
+size_t hetrd_panel_bytes(int n, int nprob);
+// digit tiles (row exponents: (n - 1) nprob ints)
 size_t hetrd_digits_bytes(int n, int nprob, int digits);
 cudaError_t launch_hetrd_digits(int n, int nprob, const int32_t* size, const z64* A, int ld, long long strideA, int i0,
                                 void* dig, int* erow, int digits, cudaStream_t st);
