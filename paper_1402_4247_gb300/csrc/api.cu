@@ -187,6 +187,8 @@ struct GenEigPlan {
   size_t oScr2, oOz2;
   // per problem: the second Newton-Schulz step's flag and column count
   size_t oNs2, oNc2;
+  // Cholesky route of the overlap: failures, norms, orders left for Eigen_HH
+  size_t oCf, oCp, oCs;
   size_t bytes;
 };
 
@@ -256,6 +258,9 @@ GenEigPlan plan_gen_eig(int n, int nprob, int nSe, bool use_tc, int B2, bool spl
   W.oOz2 = P.take<char>(split && use_tc ? zgemm_oz_workspace(np2, dmax) : 1);
   W.oNs2 = P.take<int>(nmax);
   W.oNc2 = P.take<int32_t>(nmax);
+  W.oCf = P.take<int>(nSe);
+  W.oCp = P.take<double>(chol_part_doubles(n, nSe));
+  W.oCs = P.take<int32_t>(nSe);
   W.bytes = P.off;
   return W;
 }
@@ -308,7 +313,8 @@ struct Q2Ref {
 cudaError_t backtransform_blocked(nao_ctx* ctx, int n, int nprob, const int32_t* size, const int32_t* ncols, const z64* A,
                                   const z64* tau, const double* Z, const double* w, int use_rsqrt, z64* U, z64* Vf,
                                   z64* tauc, z64* G, z64* T, z64* W, z64* VT, void* ozws, cudaStream_t st,
-                                  int digits, int lowest, int off = 1, const Q2Ref* q2 = nullptr) {
+                                  int digits, int lowest, int off = 1, const Q2Ref* q2 = nullptr,
+                                  const int32_t* on = nullptr) {
   // blocks of 128 reflectors; up to 64 reflectors take one block of 64 (T's FP64 work falls
   // eightfold, and nothing has to be joined)
   const int nb = n - off <= NAO_WY_T ? NAO_WY_T : NAO_WY_NB;
@@ -331,7 +337,7 @@ cudaError_t backtransform_blocked(nao_ctx* ctx, int n, int nprob, const int32_t*
   for (int j = 0; j < nblk; ++j) {  // Gram matrices of all blocks
     const int R0 = j * nb + off, rows = n - R0;
     const z64* Vj = Vf + R0 + (size_t)j * nb * n;  // V_j(r, c) at Vj[r + c n]
-    GemmDims dg{nb, nb, rows, nullptr, nullptr, nullptr, 0};
+    GemmDims dg{nb, nb, rows, nullptr, nullptr, nullptr, 0, 0, on};
     e = run_zgemm(ctx, "backtransform", nprob, dg, 1.0, GemmOperand{Vj, svf, n, 1, 1, nullptr},
                   GemmOperand{Vj, svf, 1, n, 0, nullptr}, 0.0, G + (size_t)j * nprob * snb2, snb2, nb, 1, ozws,
                   st, digits);
@@ -355,7 +361,7 @@ cudaError_t backtransform_blocked(nao_ctx* ctx, int n, int nprob, const int32_t*
   }
   for (int j = 0; j < nblk; ++j) {  // VT_j = V_j T_j (rows x nb; T_j upper triangular, row-major)
     const int R0 = j * nb + off, rows = n - R0;
-    GemmDims dv{rows, nb, nb, nullptr, nullptr, nullptr, 0};
+    GemmDims dv{rows, nb, nb, nullptr, nullptr, nullptr, 0, 0, on};
     e = run_zgemm(ctx, "backtransform", nprob, dv, 1.0, GemmOperand{Vf + R0 + (size_t)j * nb * n, svf, 1, n, 0, nullptr},
                   GemmOperand{T + (size_t)j * nprob * snb2, snb2, nb, 1, 0, nullptr}, 0.0,
                   VT + R0 + (size_t)j * nb * n, svf, 1, n, ozws, st, digits);
@@ -366,11 +372,11 @@ cudaError_t backtransform_blocked(nao_ctx* ctx, int n, int nprob, const int32_t*
     if (rows <= 0) continue;
     const z64* Vj = Vf + R0 + (size_t)j * nb * n;
     const z64* VTj = VT + R0 + (size_t)j * nb * n;
-    GemmDims dw{nb, n, rows, nullptr, ncols, nullptr, 0};
+    GemmDims dw{nb, n, rows, nullptr, ncols, nullptr, 0, 0, on};
     e = run_zgemm(ctx, "backtransform", nprob, dw, 1.0, GemmOperand{Vj, svf, n, 1, 1, nullptr},
                   GemmOperand{U + R0, snn, 1, n, 0, nullptr}, 0.0, W, snbn, n, 1, ozws, st, digits);
     if (e != cudaSuccess) return e;
-    GemmDims du{rows, n, nb, nullptr, ncols, nullptr, 0};
+    GemmDims du{rows, n, nb, nullptr, ncols, nullptr, 0, 0, on};
     e = run_zgemm(ctx, "backtransform", nprob, du, -1.0, GemmOperand{VTj, svf, 1, n, 0, nullptr},
                   GemmOperand{W, snbn, n, 1, 0, nullptr}, 1.0, U + R0, snn, 1, n, ozws, st, digits);
     if (e != cudaSuccess) return e;
@@ -386,7 +392,8 @@ cudaError_t backtransform_blocked(nao_ctx* ctx, int n, int nprob, const int32_t*
 // (NAO_HT_DIGITS_FP64, or NAO_HT_DIGITS_MIXED for the H' reduction of the mixed mode).
 cudaError_t hetrd_blocked(nao_ctx* ctx, int n, int nprob, const int32_t* size, z64* A, double* d, double* e, z64* tau,
                           z64* VW, void* ozws, cudaStream_t st, int digits, void* dig, int* erow,
-                          void* md, int panel_digits = NAO_HT_DIGITS_FP64, int cluster_nprob = 0) {
+                          void* md, int panel_digits = NAO_HT_DIGITS_FP64, int cluster_nprob = 0,
+                          const int32_t* on = nullptr) {
   // exact integer matrix-vector products with the tensor-core method; FP64 FMAs otherwise
   // (up to the order whose digit words still fit in a block's shared memory)
   const bool use_dig = ctx->gemm_method == NAO_GEMM_TC && dig != nullptr && hetrd_digits_fit(n, panel_digits);
@@ -415,7 +422,7 @@ cudaError_t hetrd_blocked(nao_ctx* ctx, int n, int nprob, const int32_t* size, z
     const int r0 = i0 + NB;
     if (r0 >= n) break;
     const int rows = n - r0;
-    GemmDims dd{rows, rows, 2 * NB, nullptr, nullptr, nullptr, 1};
+    GemmDims dd{rows, rows, 2 * NB, nullptr, nullptr, nullptr, 1, 0, on};
     // [V | W] (rows r0..) times [W | V]^H; VW holds the panel's columns column-major
     z64* VWr = VW + (size_t)nprob * svw;
     err = run_zgemm(ctx, "hetrd_update", nprob, dd, -1.0, GemmOperand{VWr + (size_t)r0 * 3 * NB, svw, 3 * NB, 1, 0, nullptr},
@@ -502,9 +509,9 @@ cudaError_t hetrd_two_stage(nao_ctx* ctx, int n, int nprob, const int32_t* size,
 // of it are far below Z's own rounding.  Otherwise the FP32 SIMT correction into Z2.
 // Returns the array that holds the result.
 double* ns_correct(nao_ctx* ctx, int n, int nprob, const int32_t* size, const int32_t* ncols, double* Z, double* G,
-                   double* Z2, void* ozws, cudaStream_t st, cudaError_t* err) {
+                   double* Z2, void* ozws, cudaStream_t st, cudaError_t* err, const int32_t* on = nullptr) {
   const long long snn = (long long)n * n;
-  const GemmDims d{n, n, n, size, ncols, ncols};
+  const GemmDims d{n, n, n, size, ncols, ncols, 0, 0, on};
   if (ctx->gemm_method == NAO_GEMM_TC && ozws && dgemm_oz_supported(d)) {
     NaoStage stage_(ctx, "ortho_ns", st, 4);
     *err = launch_sym_minus_identity(n, nprob, ncols, G, n, snn, st);
@@ -541,11 +548,50 @@ double* ns_second(nao_ctx* ctx, int n, int nprob, const int32_t* size, const int
     if (*err != cudaSuccess) return Zo;
     nc = ncols2;
   }
-  const GemmDims d{n, n, n, nc, nc, size, 1};
+  const GemmDims d{n, n, n, nc, nc, size, 1, 0, tc ? ns2 : nullptr};
   *err = run_dgemm(ctx, "ortho_ns", nprob, d, 1.0, GemmOperand{Zo, snn, n, 1, 0, nullptr},
                    GemmOperand{Zo, snn, 1, n, 0, nullptr}, 0.0, G, snn, 1, n, ozws, st);
   if (*err != cudaSuccess) return Zo;
-  return ns_correct(ctx, n, nprob, size, nc, Zo, G, Zo == Z ? Z2 : Z, ozws, st, err);
+  return ns_correct(ctx, n, nprob, size, nc, Zo, G, Zo == Z ? Z2 : Z, ozws, st, err, tc ? ns2 : nullptr);
+}
+
+// Part 2 without Eigen_HH (csrc/chol.cu): X = L^{-H} of every overlap matrix, S given full in X;
+// size_eff says which of them still need Eigen_HH(S).  Y, fail, part: scratch.  digits: planes of the
+// products (the mixed mode's X is as accurate as its back-transformations).
+cudaError_t overlap_cholesky(nao_ctx* ctx, int n, int nS, const int32_t* size, const z64* S, z64* X, double s_cut, z64* Y,
+                             int* fail, double* part, int32_t* size_eff, void* ozws, cudaStream_t st, int digits) {
+  const long long snn = (long long)n * n;
+  // 32 columns per step while a step is bound by its launches and its diagonal block (29 us of FP64
+  // at 32 columns, 155 us at 64), 64 once the passes over the trailing matrices (~27 ns per
+  // 1000 entries) cost more than that
+  const int B = (long long)nS * n * n > 3000000 ? 64 : 32;
+  cudaError_t e;
+  {
+    NaoStage stage_(ctx, "overlap_chol", st, 1);
+    e = launch_herm_fill(n, nS, S, snn, nullptr, X, n, snn, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(fail, 0, sizeof(int) * (size_t)nS, st);
+    if (e != cudaSuccess) return e;
+  }
+  for (int j0 = 0; j0 < n; j0 += B) {
+    const int w = n - j0 < B ? n - j0 : B, rest = n - j0 - w;
+    z64* P = X + (size_t)j0 * n;  // the block column
+    {
+      NaoStage stage_(ctx, "overlap_chol", st, 1);
+      e = launch_chol_diag(B, n, nS, size, X, snn, j0, Y, fail, st);
+      if (e != cudaSuccess) return e;
+    }
+    e = run_zgemm(ctx, "overlap_chol", nS, GemmDims{n, w, w, nullptr, nullptr, nullptr, 0}, 1.0,
+                  GemmOperand{P, snn, 1, n, 0, nullptr}, GemmOperand{Y, (long long)B * B, 1, B, 1, nullptr}, 0.0, P, snn, 1,
+                  n, ozws, st, digits);  // times Y^H, in place (the operands are split first)
+    if (e != cudaSuccess) return e;
+    if (rest == 0) break;
+    e = run_zgemm(ctx, "overlap_chol", nS, GemmDims{n, rest, w, nullptr, nullptr, nullptr, 0}, -1.0,
+                  GemmOperand{P, snn, 1, n, 0, nullptr}, GemmOperand{P + j0 + w, snn, n, 1, 1, nullptr}, 1.0,
+                  X + (size_t)(j0 + w) * n, snn, 1, n, ozws, st, digits);
+    if (e != cudaSuccess) return e;
+  }
+  NaoStage stage_(ctx, "overlap_chol", st, 2);
+  return launch_chol_decide(n, nS, size, X, S, snn, s_cut, part, fail, size_eff, st);
 }
 
 bool is_device_ptr(const void* p) {
@@ -859,28 +905,45 @@ int nao_gen_eig_sized(nao_ctx* ctx, int n, int nprob, const nao_c128* H, const n
   NAO_STAGE("herm_fill", 1, launch_herm_fill(n, nSe, (const z64*)S, snn, nullptr, AS, n, snn, st));
   // s_size (nullable): the order of each overlap matrix; the leading s_size x s_size block
   // holds it, the rest of the n x n array is zero, and the chain keeps to the block
+  // X by Cholesky where nothing is cut (csrc/chol.cu); sz then holds the orders of the matrices
+  // left for Eigen_HH(S), 0 for the others.  The alternatives that are settings of Eigen_HH, and
+  // an iteration cap below the default, keep all of it; so do the mixed mode's Ritz sweeps and raw
+  // results (one sweep's convergence is stated against the orthonormality error of that route's
+  // vectors, which X from the Cholesky factor makes smaller than their error along H').
+  const bool chol = use_tc && (!mixed || ctx->refine_sweeps == 0) && B2 == 0 && !ctx->cfg.mrrr_all && ctx->cfg.overlap_mrrr &&
+                    ctx->cfg.inverse_iteration_max >= NAO_INV_ITER_DEFAULT;
+  const int32_t* sz = s_size;
+  const int32_t* on = nullptr;
+  if (chol) {
+    int32_t* se = (int32_t*)(ws + W.oCs);
+    NAO_CUDA_TRY(ctx, overlap_cholesky(ctx, n, nSe, s_size, (const z64*)S, X, s_cut, Tw, (int*)(ws + W.oCf),
+                                       (double*)(ws + W.oCp), se, ozws, st, dig));
+    sz = on = se;
+  }
   if (B2 > 0)
-    NAO_CUDA_TRY(ctx, hetrd_two_stage(ctx, n, nSe, s_size, AS, dS, eS, tauS, sbr, B2, ozws, st, NAO_OZ_DIGITS_FP64));
+    NAO_CUDA_TRY(ctx, hetrd_two_stage(ctx, n, nSe, sz, AS, dS, eS, tauS, sbr, B2, ozws, st, NAO_OZ_DIGITS_FP64));
   else
-    NAO_CUDA_TRY(ctx, hetrd_blocked(ctx, n, nSe, s_size, AS, dS, eS, tauS, VWp, ozws, st, NAO_OZ_DIGITS_FP64, digp, erowp, mdp));
+    NAO_CUDA_TRY(ctx, hetrd_blocked(ctx, n, nSe, sz, AS, dS, eS, tauS, VWp, ozws, st, NAO_OZ_DIGITS_FP64, digp, erowp, mdp,
+                                    NAO_HT_DIGITS_FP64, 0, on));
   const int mrrr_s = ctx->cfg.mrrr_all ? 2 : ctx->cfg.overlap_mrrr, mrrr_h = ctx->cfg.mrrr_all ? 2 : 0;
   NAO_STAGE("stein", mrrr_s ? 5 : 4,
-            launch_stein(n, nSe, s_size, dS, eS, n, wS, Z, n, snn, scr, stS, nullptr, n,
+            launch_stein(n, nSe, sz, dS, eS, n, wS, Z, n, snn, scr, stS, nullptr, n,
                          ctx->cfg.inverse_iteration_max, mrrr_s, st, ns2f));
-  NAO_STAGE("misc", 1, launch_count_kept(n, nSe, s_size, wS, n, s_cut, mS, stS, st));
+  NAO_STAGE("misc", 1, launch_count_kept(n, nSe, sz, wS, n, s_cut, mS, stS, st));
   double* Zo = Z2;  // the Newton-Schulz result (Z itself on the tensor-core method)
   {  // one Newton-Schulz step: Z (3I - Z^T Z)/2 = Z - Z (Z^T Z - I)/2
-    GemmDims d{n, n, n, s_size, s_size, s_size, 1};
+    GemmDims d{n, n, n, sz, sz, sz, 1, 0, on};
     NAO_CUDA_TRY(ctx, run_dgemm(ctx, "ortho_ns", nSe, d, 1.0, GemmOperand{Z, snn, n, 1, 0, nullptr},
                                 GemmOperand{Z, snn, 1, n, 0, nullptr}, 0.0, G, snn, 1, n, ozws, st));
     cudaError_t e = cudaSuccess;
-    Zo = ns_correct(ctx, n, nSe, s_size, s_size, Z, G, Z2, ozws, st, &e);
+    Zo = ns_correct(ctx, n, nSe, sz, sz, Z, G, Z2, ozws, st, &e, on);
     NAO_CUDA_TRY(ctx, e);
-    Zo = ns_second(ctx, n, nSe, s_size, s_size, ns2f, nc2, Zo, Z, Z2, G, ozws, st, &e);
+    Zo = ns_second(ctx, n, nSe, sz, sz, ns2f, nc2, Zo, Z, Z2, G, ozws, st, &e);
     NAO_CUDA_TRY(ctx, e);
   }
-  NAO_CUDA_TRY(ctx, backtransform_blocked(ctx, n, nSe, s_size, mS, AS, tauS, Zo, wS, 1, X, Vf, tauc, Gw, Tw, Ww, VTw,
-                                          ozws, st, dig, 0, hoff, q2));
+  NAO_CUDA_TRY(ctx, backtransform_blocked(ctx, n, nSe, sz, mS, AS, tauS, Zo, wS, 1, X, Vf, tauc, Gw, Tw, Ww, VTw,
+                                          ozws, st, dig, 0, hoff, q2, on));
+  if (chol) NAO_STAGE("misc", 1, launch_chol_counts(n, nSe, s_size, on, mS, stS, st));
   {
     NaoStage stage_(ctx, "misc", st, 1);
     gather_m_kernel<<<(nprob + 127) / 128, 128, 0, st>>>(nprob, s_of_prob, mS, stS, nb, mP, nbP, stP);

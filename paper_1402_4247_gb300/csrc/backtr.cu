@@ -136,7 +136,7 @@ __global__ void extract_v_kernel(int n, const int32_t* __restrict__ size, const 
   const int m = size ? size[p] : n;
   const int i = blockIdx.y;  // column
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= n || i >= ncolv) return;
+  if (r >= n || i >= ncolv || m == 0) return;  // (order 0: nothing reads the result)
   const z64* A = Abase + (size_t)p * strideA;
   z64 val = zmk(0.0, 0.0);
   if (i < m - off) {
@@ -157,7 +157,7 @@ __global__ void init_u_kernel(int n, const int32_t* __restrict__ size, const int
   const int nc = ncols ? ncols[p] : m;
   const int c = blockIdx.y;
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= n) return;
+  if (r >= n || m == 0) return;  // (order 0: U is left alone)
   double v = 0.0;
   if (c < nc && r < m) v = Zbase[(size_t)p * strideZ + (size_t)(lowest ? c : m - nc + c) * ldz + r];
   Ubase[(size_t)p * strideU + (size_t)c * ldu + r] = zmk(v, 0.0);

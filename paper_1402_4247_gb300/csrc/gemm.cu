@@ -42,7 +42,7 @@ gemm_kernel(GemmDims dims, T alpha, GemmOperand A, GemmOperand B, T beta, T* __r
   const int Nn = dims.Np ? dims.Np[p] : dims.N;
   const int K = gemm_k(dims, p);
   const int i0 = blockIdx.y * BM, j0 = blockIdx.x * BN;
-  if (i0 >= M || j0 >= Nn) return;
+  if (i0 >= M || j0 >= Nn || (dims.on && !dims.on[p])) return;
   if (dims.lower && j0 > i0 + BM - 1) return;  // tile entirely above the diagonal
   const T* Ap = (const T*)A.ptr + (size_t)(A.map ? A.map[p] : p) * A.bs;
   const T* Bp = (const T*)B.ptr + (size_t)(B.map ? B.map[p] : p) * B.bs;

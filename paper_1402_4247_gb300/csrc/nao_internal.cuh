@@ -228,6 +228,17 @@ cudaError_t launch_stein(int n, int nprob, const int32_t* size, const double* d,
 // ns2 (nullable, [nprob]): set to 1 for a problem whose vectors need a second Newton-Schulz
 // step (a gap in [1e-11, 1e-9) |T|_1, where inverse iteration leaves overlaps up to ~1e-5)
 
+// Overlap chain by Cholesky (csrc/chol.cu): the diagonal block of one step (B = 32 or 64 columns
+// from j0; Y: B x B per matrix; fail[p] set where a pivot is not positive), the decision per matrix
+// (size_eff: 0 done, else its order; part: chol_part_doubles), the kept counts of those done.
+cudaError_t launch_chol_diag(int B, int n, int nprob, const int32_t* size, z64* X, long long sX, int j0, z64* Y, int* fail,
+                             cudaStream_t st);
+size_t chol_part_doubles(int n, int nprob);
+cudaError_t launch_chol_decide(int n, int nprob, const int32_t* size, z64* X, const z64* S, long long sX, double s_cut,
+                               double* part, const int* fail, int32_t* size_eff, cudaStream_t st);
+cudaError_t launch_chol_counts(int n, int nprob, const int32_t* size, const int32_t* size_eff, int32_t* m, int32_t* status,
+                               cudaStream_t st);
+
 // Blocked (compact WY) back-transformation helpers, see backtr.cu.
 constexpr int NAO_WY_NB = 128;
 constexpr int NAO_WY_T = 64;  // T_j is formed in diagonal blocks of this order, joined by products
@@ -261,6 +272,7 @@ struct GemmDims {
   int lower = 0;                        // 1: only output tiles that meet the lower triangle
   int k0 = 0;                           // contraction chunk start: with Kp, problem p's length
                                         // is min(max(Kp[p] - k0, 0), K)
+  const int32_t* on = nullptr;          // problems with on[p] = 0 are left out (nullable: all)
 };
 // per-problem contraction length of a (possibly chunked) product
 __host__ __device__ inline int gemm_k(const GemmDims& d, int p) {

@@ -191,6 +191,7 @@ __global__ void __launch_bounds__(256) oz_split(int nprob, GemmDims dims, GemmOp
   constexpr int TB = TR * OZ_BK * 2;                  // bytes per plane tile
   constexpr int SCALE0 = IS_B ? 30 : 0;               // plane s holds d_s 2^{SCALE0 - DB s}
   const int p = blockIdx.y;
+  if (dims.on && !dims.on[p]) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int lr = (lane & 7) + 8 * (lane >> 4);
   const int kh = (lane >> 3) & 1;
@@ -395,6 +396,7 @@ oz_gemm_kernel(int nprob, GemmDims dims, double alpha, double beta, const __nv_b
   const int N = dims.Np ? dims.Np[p] : dims.N;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   // uniform early exits (before any barrier or allocation)
+  if (dims.on && !dims.on[p]) return;
   const int CPT = REAL ? BN : BN / 2;  // output columns per tile
   if (rb * OZ_BM >= M || cb * CPT >= N) return;
   if (dims.lower && cb * CPT > rb * OZ_BM + OZ_BM - 1) return;
