@@ -172,12 +172,12 @@ constexpr int NAO_HT_NB = 32;
 // 6 (46 bits: the H' reduction of the mixed mode); 0 selects the FP64 form.
 constexpr int NAO_HT_DIGITS_FP64 = 8;
 constexpr int NAO_HT_DIGITS_MIXED = 6;
-// FP64 form (csrc/hetrd.cu)
+// FP64 form (csrc/hetrd_fp64.cu)
 int hetrd_cluster_size(int n, int nprob, int num_sms);
 cudaError_t launch_hetrd_panel(int n, int nprob, const int32_t* size, z64* A, int ld, long long strideA, double* d,
                                double* e, z64* tau, long long strideV, z64* VW, long long strideVW, int i0, int cluster,
                                z64* VWr, cudaStream_t st);
-// digit form (csrc/hetrd_mma.cu).  dig / erow: 8-bit digit tiles of the trailing matrix and the
+// digit form (csrc/hetrd.cu).  dig / erow: 8-bit digit tiles of the trailing matrix and the
 // rows' exponents, made by launch_hetrd_digits for this panel with the same digit count
 bool hetrd_digits_fit(int n, int digits);  // its shared memory fits a block at order n
 int hetrd_mma_cluster_size(int n, int nprob, int num_sms, int digits);
