@@ -20,20 +20,23 @@
 //        one thread per queue entry, so that its warps are full.
 // * Eigenvectors (kernel 2, same block split): inverse iteration with a partially pivoted LU
 //   of T - lambda I (tiny pivots perturbed to eps |T|), a scaled right-hand side, the growth
-//   test |x|_inf >= sqrt(0.1/blocksize) within `maxits` solves plus two extra solves, and
-//   modified Gram-Schmidt against the earlier members of a tight cluster (gap < 1e-11 |T|_1;
-//   1e-9 |T|_1 when kernel 0 runs), whose leader walks the cluster in order.  Wider
-//   near-degeneracies leave overlaps of order eps|T|/gap, which the caller removes with
-//   Newton-Schulz steps Z <- Z (3I - Z^T Z)/2 (each squares them): one step for gaps
-//   >= 1e-9 |T|_1 (overlaps <= ~1e-7), a second one for the problems flagged in ns2[] because
-//   a gap lies in [1e-11, 1e-9) |T|_1 (overlaps <= ~1e-5).
-//   A tight cluster of more than BIG members (the near-null spectrum of an ill-conditioned
-//   overlap matrix can chain hundreds) is handed to kernel 3: one block per cluster, the
-//   same iteration with the reorthogonalisation done by the whole block (classical
-//   Gram-Schmidt applied twice) while one thread runs the tridiagonal solves.  A chain can
-//   span far more than the tight band; a member is re-orthogonalised only against the
-//   finished members within the band of its own eigenvalue (the others overlap it by at
-//   most eps|T| over the band, which the Newton-Schulz steps remove).
+//   test |x|_inf >= sqrt(0.1/blocksize) within `maxits` solves plus one or two extra solves, one
+//   thread per eigenvalue whether or not it has close neighbours.  Wider near-degeneracies leave
+//   overlaps of order eps|T|/gap, which the caller removes with Newton-Schulz steps
+//   Z <- Z (3I - Z^T Z)/2 (each squares them): one step for gaps >= 1e-9 |T|_1 (overlaps <= ~1e-7),
+//   a second one for the problems flagged in ns2[] because a gap lies in [1e-11, 1e-9) |T|_1
+//   (overlaps <= ~1e-5).
+//   The members of a tight cluster (gap < 1e-11 |T|_1; 1e-9 |T|_1 when kernel 0 runs) are then
+//   orthogonalised by kernel 3, one block per cluster, in ascending order (classical
+//   Gram-Schmidt applied twice against the finished members): two vectors with a gap g overlap by at
+//   most ~eps|T|/g, so taking one out of the other changes its residual by overlap x g, of order
+//   eps|T| again.  A member that loses nearly all of its norm (its random start fell into the
+//   others' span) is iterated again from another start with the orthogonalisation inside
+//   the iteration, its solves in one thread.  A chain can span far more than the tight band; a member
+//   is orthogonalised only against the finished members within the band of its own
+//   eigenvalue (the others overlap it by at most eps|T| over the band, which the Newton-Schulz
+//   steps remove).  (Before, one thread walked each cluster of up to 32 members and ran all
+//   solves of larger ones: n = 600, 8 problems with 12 null directions each, 85 -> 18 ms.)
 // * Output: eigenvalues ascending (across blocks), eigenvectors in matching columns,
 //   unit 2-norm, largest component positive.  All loops are bounded.
 #include <cfloat>
@@ -56,7 +59,7 @@ constexpr double TIGHT_GS = 1e-11;  // ...and below this, Gram-Schmidt (without 
                                     // them, Gram-Schmidt starts at TIGHT: the big clusters that the
                                     // wider band chains go to MRRR, which needs no serial walk)
 constexpr int NARR = 6;           // scratch arrays per eigenvalue: L, U0inv, U1, U2, PIV, X
-constexpr int BIG = 32;           // tight clusters with more members go to stein_cluster_kernel
+constexpr int BIG = 32;           // tight clusters with more members take kernel 0's vectors when it runs
 constexpr int NEWTON_MAX = 6;     // Newton steps on an isolated eigenvalue before it is queued
 constexpr int BQ_LANES = 4;       // lanes per queued eigenvalue in the FP64 bisection (multisection)
 
@@ -477,11 +480,10 @@ stein_vec_kernel(int n, const int32_t* __restrict__ size, const double* __restri
   __syncthreads();
   if (j < m) {
     const int b0 = bst[j], b1 = ben[j];
-    const bool leader = !(j > b0 && w[j] - w[j - 1] < tight);
-    int jend = j + 1;
-    if (leader)
+    const bool close_lo = j > b0 && w[j] - w[j - 1] < tight, close_hi = j + 1 < b1 && w[j + 1] - w[j] < tight;
+    if (close_hi && !close_lo) {  // the first member lists the cluster for kernel 3
+      int jend = j + 2;
       while (jend < b1 && w[jend] - w[jend - 1] < tight) ++jend;
-    if (leader && jend - j > BIG) {  // hand the cluster to kernel 3
       const int slot = atomicAdd(&biglist[0], 1);
       if (slot < bigcap) {
         biglist[1 + 3 * slot] = p;
@@ -490,7 +492,8 @@ stein_vec_kernel(int n, const int32_t* __restrict__ size, const double* __restri
       } else {
         s_fail = 1;
       }
-    } else if (leader) {
+    }
+    {
       const int bs = b1 - b0;
       double* __restrict__ Lr = scr + 0 * nn;
       double* __restrict__ U0i = scr + 1 * nn;
@@ -498,35 +501,25 @@ stein_vec_kernel(int n, const int32_t* __restrict__ size, const double* __restri
       double* __restrict__ U2 = scr + 3 * nn;
       double* __restrict__ PV = scr + 4 * nn;
       double* __restrict__ X = scr + 5 * nn;
-      const int sl = j;  // scratch column of this leader
+      const int sl = j;  // scratch column
 #define AT(arr, i) arr[(size_t)(i) * n + sl]
-      double lamprev = 0.0;
-      for (int q = j; q < jend; ++q) {
-        // rank of slot q (recomputed: members of a cluster may belong to other threads' slots)
+      const int q = j;
+      do {
         const double wq = w[q];
-        int rq = 0;
+        int rq = 0;  // rank in the global ascending order
         for (int t = 0; t < m; ++t) {
           const double wt = w[t];
           rq += (wt < wq) || (wt == wq && t < q);
         }
-        if (rq >= nv) break;  // members ascend: the rest of the cluster is not wanted either
+        if (rq >= nv) break;
         const int* dn = mdone ? mdone + (size_t)p * n : nullptr;
-        if (dn && dn[q]) {  // an MRRR vector (kernel 0) is already in Z
-          lamprev = wq;
-          continue;
-        }
+        if (dn && dn[q]) break;  // an MRRR vector (kernel 0) is already in Z
         double* zc = Z + (size_t)rq * ldz;
         if (bs == 1) {
           for (int i = 0; i < m; ++i) zc[i] = (i == b0) ? 1.0 : 0.0;
-          lamprev = wq;
-          continue;
+          break;
         }
-        double lam = wq;
-        if (q > j) {
-          const double pertol = 10.0 * fabs(eps * lam);
-          if (lam - lamprev < pertol) lam = lamprev + pertol;
-        }
-        lamprev = lam;
+        const double lam = wq;
         // LU with partial pivoting of T[b0:b1) - lam I
         double al = d[b0] - lam, be = e[b0];
         for (int k = b0; k < b1 - 1; ++k) {
@@ -602,16 +595,6 @@ stein_vec_kernel(int n, const int32_t* __restrict__ size, const double* __restri
             x2 = x1v;
             x1v = xv;
           }
-          for (int t = j; t < jend; ++t) {  // reorthogonalise against the cluster's finished members
-            if (t == q || (t > q && !(dn && dn[t]))) continue;
-            const double wt = w[t];
-            int rt = 0;
-            for (int u = 0; u < m; ++u) rt += (w[u] < wt) || (w[u] == wt && u < t);
-            const double* zt = Z + (size_t)rt * ldz;
-            double dot = 0.0;
-            for (int i = b0; i < b1; ++i) dot = fma(AT(X, i), zt[i], dot);
-            for (int i = b0; i < b1; ++i) AT(X, i) = fma(-dot, zt[i], AT(X, i));
-          }
           double xinf = 0.0;
           bool finite = true;
           x1 = 0.0;
@@ -625,7 +608,7 @@ stein_vec_kernel(int n, const int32_t* __restrict__ size, const double* __restri
           if (its > maxits && nrmchk == 0) break;
           if (xinf < sqrt(0.1 / bs)) continue;
           ++nrmchk;
-          if (nrmchk < (jend - j > 1 ? EXTRA : EXTRA_ISOLATED) + 1) continue;
+          if (nrmchk < (close_lo || close_hi ? EXTRA : EXTRA_ISOLATED) + 1) continue;
           ok = true;
           break;
         }
@@ -644,7 +627,7 @@ stein_vec_kernel(int n, const int32_t* __restrict__ size, const double* __restri
         if (AT(X, jmax) < 0.0) sc = -sc;
         for (int i = 0; i < m; ++i) zc[i] = (i >= b0 && i < b1) ? AT(X, i) * sc : 0.0;
         if (sc == 0.0) zc[b0 + (q - b0) % bs] = 1.0;  // keep a unit vector even on failure
-      }
+      } while (false);
 #undef AT
     }
   }
@@ -652,10 +635,11 @@ stein_vec_kernel(int n, const int32_t* __restrict__ size, const double* __restri
   if (threadIdx.x == 0 && s_fail && status) atomicExch(&status[p], NAO_E_NOCONV);
 }
 
-// ---------------------------------------------------------------- kernel 3: big tight clusters
-// One block per cluster listed by kernel 2: members in ascending order; thread 0 factors
-// T - lambda I and runs the solves (as kernel 2), the block re-orthogonalises each iterate
-// against the earlier members (classical Gram-Schmidt, twice) and takes the norms.
+// ---------------------------------------------------------------- kernel 3: tight clusters
+// One block per cluster listed by kernel 2: members in ascending order.  Kernel 2's vector is
+// orthogonalised by the block against the finished members (classical Gram-Schmidt, twice); one
+// whose norm falls below CL_KEEP is iterated anew: thread 0 factors T - lambda I and runs the
+// solves (as kernel 2), the block re-orthogonalises each iterate and takes the norms.
 __device__ __forceinline__ double block_sum1(double v, double* red) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
 #pragma unroll
@@ -680,6 +664,7 @@ __device__ __forceinline__ double block_max1(double v, double* red) {
 }
 
 constexpr int SC_THREADS = 256;
+constexpr double CL_KEEP = 1e-2;  // (1 - norm^2 is the share of the others: rounding grows by 1 / CL_KEEP at most)
 
 __global__ void __launch_bounds__(SC_THREADS, 1)
 stein_cluster_kernel(int n, const int32_t* __restrict__ size, const double* __restrict__ dbase,
@@ -751,6 +736,38 @@ stein_cluster_kernel(int n, const int32_t* __restrict__ size, const double* __re
       }
       const int sl = q;
 #define AT(arr, i) arr[(size_t)(i) * n + sl]
+      // classical Gram-Schmidt, twice, of sx against the finished members of the band
+      auto orthogonalise = [&]() {
+        __syncthreads();
+        const int nf = s_nf;
+        for (int pass = 0; pass < 2 && nf > 0; ++pass) {
+          for (int u = wid; u < nf; u += nw) {
+            const double* zt = Z + (size_t)rnk[fin[u]] * ldz;
+            double dt = 0.0;
+            for (int i = b0 + lane; i < b1; i += 32) dt = fma(sx[i], zt[i], dt);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) dt += __shfl_xor_sync(0xffffffffu, dt, o);
+            if (lane == 0) dots[u] = dt;
+          }
+          __syncthreads();
+          for (int i = b0 + tid; i < b1; i += nt) {
+            double v = sx[i];
+            for (int u = 0; u < nf; ++u) v = fma(-dots[u], Z[(size_t)rnk[fin[u]] * ldz + i], v);
+            sx[i] = v;
+          }
+          __syncthreads();
+        }
+      };
+      {
+        const double* zc = Z + (size_t)rnk[q - j] * ldz;
+        for (int i = b0 + tid; i < b1; i += nt) sx[i] = zc[i];
+      }
+      orthogonalise();
+      double a0 = 0.0;
+      for (int i = b0 + tid; i < b1; i += nt) a0 = fma(sx[i], sx[i], a0);
+      const double kept = block_sum1(a0, red);
+      const bool again = !(kept >= CL_KEEP * CL_KEEP && kept <= 4.0);  // uniform (NaN: again)
+      if (again) {
       if (tid == 0) {  // LU with partial pivoting of T[b0:b1) - lam I (as kernel 2)
         double lam = w[q];
         if (q > j) {
@@ -832,24 +849,7 @@ stein_cluster_kernel(int n, const int32_t* __restrict__ size, const double* __re
           }
         }
         __syncthreads();
-        const int nf = s_nf;  // (published by the barriers above)
-        for (int pass = 0; pass < 2 && nf > 0; ++pass) {
-          for (int u = wid; u < nf; u += nw) {
-            const double* zt = Z + (size_t)rnk[fin[u]] * ldz;
-            double dt = 0.0;
-            for (int i = b0 + lane; i < b1; i += 32) dt = fma(sx[i], zt[i], dt);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) dt += __shfl_xor_sync(0xffffffffu, dt, o);
-            if (lane == 0) dots[u] = dt;
-          }
-          __syncthreads();
-          for (int i = b0 + tid; i < b1; i += nt) {
-            double v = sx[i];
-            for (int u = 0; u < nf; ++u) v = fma(-dots[u], Z[(size_t)rnk[fin[u]] * ldz + i], v);
-            sx[i] = v;
-          }
-          __syncthreads();
-        }
+        orthogonalise();
         double am = 0.0;
         bool fin = true;
         for (int i = b0 + tid; i < b1; i += nt) {
@@ -867,6 +867,9 @@ stein_cluster_kernel(int n, const int32_t* __restrict__ size, const double* __re
         break;
       }
       if (!ok) fail = true;
+      } else {
+        lamprev = w[q];
+      }
       // normalise, sign: largest component positive (first of equal magnitude)
       double a2 = 0.0, big = 0.0;
       int jm = b1;
@@ -1159,8 +1162,8 @@ mrrr_vec_kernel(int n, const int32_t* __restrict__ size, const double* __restric
 }  // namespace
 
 // scratch: NARR n^2 doubles per problem, the eigenvalue slots (n per problem), and the
-// big-cluster list (count + 3 ints per cluster, at most n / (BIG + 1) clusters per problem)
-static int big_capacity(int n, int nprob) { return nprob * (n / (BIG + 1) + 1); }
+// cluster list (count + 3 ints per cluster, at most n / 2 clusters per problem)
+static int big_capacity(int n, int nprob) { return nprob * (n / 2 + 1); }
 
 size_t stein_scratch_doubles(int n, int nprob) {
   // the bisection queue (5 n + 1 doubles per problem, + 1) fits in the first NARR n^2 per
