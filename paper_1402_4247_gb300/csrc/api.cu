@@ -399,11 +399,19 @@ cudaError_t hetrd_blocked(nao_ctx* ctx, int n, int nprob, const int32_t* size, z
   const bool use_dig = ctx->gemm_method == NAO_GEMM_TC && dig != nullptr && hetrd_digits_fit(n, panel_digits);
   const int pd = use_dig ? panel_digits : 0;
   const int NB = NAO_HT_NB;
+  const long long snn = (long long)n * n;
   // cluster size from the number of matrices that share the GPU (cluster_nprob: a concurrent
   // launch's matrices included)
   const int np = cluster_nprob > 0 ? cluster_nprob : nprob;
+  if (use_dig) {  // (the FP64 method keeps one form, as the second route of the tests)
+    const int cs = hetrd_small_cluster(n, np, ctx->num_sms);
+    if (cs > 0) {
+      NaoStage stage_(ctx, "hetrd", st, 1);
+      return launch_hetrd_small(n, nprob, size, A, n, snn, d, e, tau, n, cs, st);
+    }
+  }
   const int cl = use_dig ? hetrd_mma_cluster_size(n, np, ctx->num_sms, pd) : hetrd_cluster_size(n, np, ctx->num_sms);
-  const long long snn = (long long)n * n, svw = (long long)n * 3 * NB;
+  const long long svw = (long long)n * 3 * NB;
   for (int i0 = 0; i0 < n; i0 += NB) {
     cudaError_t err = cudaSuccess;
     if (use_dig) {

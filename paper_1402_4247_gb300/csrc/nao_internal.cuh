@@ -177,6 +177,11 @@ int hetrd_cluster_size(int n, int nprob, int num_sms);
 cudaError_t launch_hetrd_panel(int n, int nprob, const int32_t* size, z64* A, int ld, long long strideA, double* d,
                                double* e, z64* tau, long long strideV, z64* VW, long long strideVW, int i0, int cluster,
                                z64* VWr, cudaStream_t st);
+// whole reduction in one launch, FP64, the matrix in the shared memory of a cluster
+// (csrc/hetrd_small.cu); hetrd_small_cluster: blocks per matrix, 0 where it is not the faster form
+int hetrd_small_cluster(int n, int nprob, int num_sms);
+cudaError_t launch_hetrd_small(int n, int nprob, const int32_t* size, z64* A, int ld, long long strideA, double* d, double* e,
+                               z64* tau, long long strideV, int C, cudaStream_t st);
 // digit form (csrc/hetrd.cu).  dig / erow: 8-bit digit tiles of the trailing matrix and the
 // rows' exponents, made by launch_hetrd_digits for this panel with the same digit count
 bool hetrd_digits_fit(int n, int digits);  // its shared memory fits a block at order n
