@@ -934,7 +934,7 @@ int nao_gen_eig_sized(nao_ctx* ctx, int n, int nprob, const nao_c128* H, const n
     NAO_CUDA_TRY(ctx, hetrd_blocked(ctx, n, nSe, sz, AS, dS, eS, tauS, VWp, ozws, st, NAO_OZ_DIGITS_FP64, digp, erowp, mdp,
                                     NAO_HT_DIGITS_FP64, 0, on));
   const int mrrr_s = ctx->cfg.mrrr_all ? 2 : ctx->cfg.overlap_mrrr, mrrr_h = ctx->cfg.mrrr_all ? 2 : 0;
-  NAO_STAGE("stein", mrrr_s ? 5 : 4,
+  NAO_STAGE("stein", stein_launches(n, nSe, mrrr_s),
             launch_stein(n, nSe, sz, dS, eS, n, wS, Z, n, snn, scr, stS, nullptr, n,
                          ctx->cfg.inverse_iteration_max, mrrr_s, st, ns2f));
   NAO_STAGE("misc", 1, launch_count_kept(n, nSe, sz, wS, n, s_cut, mS, stS, st));
@@ -988,7 +988,7 @@ int nao_gen_eig_sized(nao_ctx* ctx, int n, int nprob, const nao_c128* H, const n
       NAO_CUDA_TRY(ctx, hetrd_blocked(ctx, n, np, h.mP, h.Hp, h.dH, h.eH, h.tauH, h.VWp, h.ozws, st, dig, h.digp,
                                       h.erowp, h.mdp, NAO_HT_DIGITS_FP64, nprob));
       const int nv_max = C ? n : 0;
-      NAO_STAGE("stein", mrrr_h ? 5 : 4, launch_stein(n, np, h.mP, h.dH, h.eH, n, h.wH, h.Z, n, snn, h.scr, h.stH,
+      NAO_STAGE("stein", stein_launches(n, np, mrrr_h), launch_stein(n, np, h.mP, h.dH, h.eH, n, h.wH, h.Z, n, snn, h.scr, h.stH,
                                                      h.nbP, nv_max, ctx->cfg.inverse_iteration_max, mrrr_h, st,
                                                      h.ns2));
       if (nv_max > 0) {
@@ -1095,7 +1095,7 @@ int nao_gen_eig_sized(nao_ctx* ctx, int n, int nprob, const nao_c128* H, const n
   const bool all_vecs = mixed && ctx->refine_sweeps >= 0;
   const int32_t* nvP = all_vecs ? mP : nbP;
   const int nv_max = (C || all_vecs) ? n : 0;
-  NAO_STAGE("stein", mrrr_h ? 5 : 4, launch_stein(n, nprob, mP, dH, eH, n, wH, Z, n, snn, scr, stH, nvP, nv_max,
+  NAO_STAGE("stein", stein_launches(n, nprob, mrrr_h), launch_stein(n, nprob, mP, dH, eH, n, wH, Z, n, snn, scr, stH, nvP, nv_max,
                                                  ctx->cfg.inverse_iteration_max, mrrr_h, st, ns2f));
   if (nv_max > 0) {
     {

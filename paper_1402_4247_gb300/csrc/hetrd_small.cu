@@ -19,12 +19,12 @@
 //    are formed by one warp and reductions run only in warps that hold rows: with every warp
 //    forming them redundantly a column took 15,000 cycles whatever n.
 // FP64 work per column and block: 12 multiply-adds per element, 6 L^2 / C cycles (L trailing rows).
-// Rule (hetrd_small_cluster): n^2 / C <= 8000 (12000 up to n = 136), where that pass costs less than
+// Rule (hetrd_small_cluster): n^2 / C <= 9000 (12000 up to n = 136), where that pass costs less than
 // the panel's longer chain (csrc/hetrd.cu).  Whole reduction, this against panels, us: n = 64, 4
 // problems 422 / 846; n = 100, 150 problems (C = 1) 1599 / 2247; n = 129, 76 problems (C = 2)
-// 1779 / 2653; n = 160, 37 problems (C = 4) 2341 / 3089; n = 211, 18 problems (C = 8) 3029 / 4194; n = 305,
-// 1 problem (C = 16) 4772 / 5595; beyond the line n = 256, 9 problems (C = 8) 4473 / 4375, n = 360, 1
-// problem (C = 16) 6786 / 6849.
+// 1779 / 2653; n = 160, 37 problems (C = 4) 2341 / 3089; n = 211, 24 problems (C = 5) 3270 / 4140; n = 305,
+// 1 problem (C = 16) 4772 / 5595; at the line n = 256, 9 problems (C = 8) 4473 / 4375, n = 360, 1 problem
+// (C = 16) 6786 / 6849.
 #include <cooperative_groups.h>
 
 #include "nao_internal.cuh"
@@ -296,7 +296,7 @@ int hetrd_small_cluster(int n, int nprob, int num_sms) {
     return 0;
   }
   for (int c = HS_MAX_CLUSTER; c > 0; c = c > 8 ? 8 : c - 1) {
-    if (n * n > c * (n <= 136 ? 12000 : 8000)) return 0;
+    if (n * n > c * (n <= 136 ? 12000 : 9000)) return 0;
     if (c > 1 && (4 * c > n || (long long)nprob * c > num_sms)) continue;
     if (small_smem(n, c).bytes > HS_SMEM_LIMIT) return 0;
     if (c == 1) return 1;

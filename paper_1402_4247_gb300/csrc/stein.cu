@@ -61,7 +61,7 @@ constexpr double TIGHT_GS = 1e-11;  // ...and below this, Gram-Schmidt (without 
 constexpr int NARR = 6;           // scratch arrays per eigenvalue: L, U0inv, U1, U2, PIV, X
 constexpr int BIG = 32;           // tight clusters with more members take kernel 0's vectors when it runs
 constexpr int NEWTON_MAX = 6;     // Newton steps on an isolated eigenvalue before it is queued
-constexpr int BQ_LANES = 4;       // lanes per queued eigenvalue in the FP64 bisection (multisection)
+constexpr int BQ_LANES = 4;       // lanes per queued eigenvalue in the FP64 bisection (multisection), at least
 
 __device__ __forceinline__ double warp_max(double v) {
 #pragma unroll
@@ -111,7 +111,14 @@ __device__ TriInfo load_tridiag(int m, const double* __restrict__ din, const dou
     red[32 + wid] = lmax;
     red[64 + wid] = lnrm;
   }
-  if (tid == 0) {  // block boundaries (serial, O(m))
+  bool cut = false;  // block boundaries: one block, or a serial pass where T splits
+  for (int i = tid; i < m - 1; i += nt) cut = cut || e[i] == 0.0;
+  if (!__syncthreads_or(cut)) {
+    for (int i = tid; i < m; i += nt) {
+      bst[i] = 0;
+      ben[i] = m;
+    }
+  } else if (tid == 0) {
     int b0 = 0;
     for (int i = 0; i < m; ++i) {
       bst[i] = b0;
@@ -396,14 +403,18 @@ __global__ void __launch_bounds__(SZ_THREADS)
 stebz_bisect_kernel(int n, const double* __restrict__ dbase, long long strideV, const double* __restrict__ e2g,
                     const double* __restrict__ tng, double* __restrict__ wslot, const int* __restrict__ qcount,
                     const int4* __restrict__ qent, const double* __restrict__ qlo, const double* __restrict__ qhi) {
-  // BQ_LANES lanes per entry: each step counts at BQ_LANES interior points of the bracket,
-  // one per lane, and keeps the sub-interval that holds the eigenvalue (log2(BQ_LANES + 1)
-  // bits per step instead of one): the dependent chain of steps, which sets this kernel's
-  // time, is ~2.3x shorter
+  // LN lanes per entry: each step counts at LN interior points of the bracket, one per lane,
+  // and keeps the sub-interval that holds the eigenvalue (log2(LN + 1) bits per step instead of
+  // one): the dependent chain of steps sets this kernel's time.  BQ_LANES, or as many more (32 at
+  // most) as leave a short queue's warps a scheduler each (608 on this GPU)
+  const int cnt = *qcount;
+  int LN = BQ_LANES;
+  while (LN < 32 && cnt * LN <= 608 * 16) LN *= 2;
   const int gt = blockIdx.x * blockDim.x + threadIdx.x;
-  const int q = gt / BQ_LANES, sub = gt % BQ_LANES;
-  if (q >= *qcount) return;  // uniform over the entry's lanes
-  const unsigned gmask = ((1u << BQ_LANES) - 1u) << ((threadIdx.x & 31) & ~(BQ_LANES - 1));
+  const int q = gt / LN, sub = gt % LN;
+  if (q >= cnt) return;  // uniform over the entry's lanes
+  const int lane0 = (threadIdx.x & 31) & ~(LN - 1);
+  const unsigned gmask = (LN == 32 ? 0xffffffffu : (1u << LN) - 1u) << lane0;
   const int4 en = qent[q];
   const int p = en.x, j = en.y, b0 = en.z, b1 = en.w, idx = j - b0;
   const double* d = dbase + (size_t)p * strideV;
@@ -415,18 +426,101 @@ stebz_bisect_kernel(int n, const double* __restrict__ dbase, long long strideV, 
     const double mid = 0.5 * (lo + hi);
     const double tol = fmax(2.0 * eps * fmax(fabs(lo), fabs(hi)), eps * tn);
     if (hi - lo <= tol || mid <= lo || mid >= hi) break;
-    const double h = (hi - lo) / (BQ_LANES + 1);
+    const double h = (hi - lo) / (LN + 1);
     const double x = lo + h * (sub + 1);
     const bool above = (x > lo && x < hi) ? sturm64_count(d, e2, b0, b1, x, tn) > idx : x >= hi;
     // the lowest point with more than idx eigenvalues below it bounds the eigenvalue from
     // above, the point before it from below (every lane forms the same bracket)
     const unsigned ab = __ballot_sync(gmask, above) & gmask;
-    const int k = ab ? __ffs(ab) - 1 - ((threadIdx.x & 31) & ~(BQ_LANES - 1)) : BQ_LANES;
+    const int k = ab ? __ffs(ab) - 1 - lane0 : LN;
     const double xk = lo + h * (k + 1), xk1 = lo + h * k;
-    if (k < BQ_LANES) hi = xk;
+    if (k < LN) hi = xk;
     if (k > 0) lo = xk1;
   }
   if (sub == 0) wslot[(size_t)p * n + j] = 0.5 * (lo + hi);
+}
+
+// Kernels 1 and 1b in one for few eigenvalues: LN lanes per eigenvalue, each step counting at LN
+// interior points of the bracket (log2(LN + 1) bits a step), in FP32 down to the bracket that FP32
+// resolves, then (widened and verified by two FP64 counts, as in kernel 1) in FP64 to the
+// tolerance of kernel 1b.  With fewer warps than schedulers the time is the chain of steps (192
+// cycles per row and FP64 count), so every lane that would be idle shortens it; launch_stein
+// takes the LN at which a warp still has a scheduler to itself.
+// Measured (tridiagonal stage with the eigenvectors, ms, before -> now): n = 568, 2 problems 5.1 -> 2.8; n = 2000,
+// 1 problem 19.1 -> 11.5; n = 129, 12 problems 0.86 -> 0.78.
+constexpr int SM_THREADS = 128;
+template <int LN>
+__global__ void __launch_bounds__(SM_THREADS)
+stebz_multi_kernel(int n, const int32_t* __restrict__ size, const double* __restrict__ dbase,
+                   const double* __restrict__ ebase, long long strideV, double* __restrict__ wslot,
+                   int32_t* __restrict__ status) {
+  extern __shared__ double smd[];
+  double* d = smd;
+  double* e = smd + n;
+  double* e2 = smd + 2 * n;
+  float* d32 = (float*)(smd + 3 * n);
+  float* e232 = d32 + n;
+  int* bst = (int*)(e232 + n);
+  int* ben = bst + n;
+  __shared__ double red[96];
+  const int p = blockIdx.y;
+  const int m = size ? size[p] : n;
+  if (m <= 0) {
+    if (blockIdx.x == 0 && threadIdx.x == 0 && status) status[p] = 0;
+    return;
+  }
+  const int gt = blockIdx.x * SM_THREADS + threadIdx.x, j = gt / LN, sub = gt % LN;
+  if ((int)(blockIdx.x * SM_THREADS) / LN >= m) return;  // uniform per block
+  const TriInfo T = load_tridiag(m, dbase + (size_t)p * strideV, ebase + (size_t)p * strideV, d, e, e2, bst, ben, red);
+  for (int i = threadIdx.x; i < m; i += SM_THREADS) {
+    d32[i] = (float)d[i];
+    e232[i] = (float)e2[i];
+  }
+  __syncthreads();
+  if (blockIdx.x == 0 && threadIdx.x == 0 && status) status[p] = 0;
+  if (j >= m) return;  // uniform over an eigenvalue's lanes
+  const int lane0 = (threadIdx.x & 31) & ~(LN - 1);
+  const unsigned gmask = (LN == 32 ? 0xffffffffu : (1u << LN) - 1u) << lane0;
+  const int b0 = bst[j], b1 = ben[j], idx = j - b0;
+  double lam;
+  if (b1 - b0 == 1) {
+    lam = d[b0];
+  } else {
+    float lo32 = (float)T.gl, hi32 = (float)T.gu;
+    const float tn32 = (float)T.tnorm;
+    for (int it = 0; it < 64; ++it) {
+      const float h = (hi32 - lo32) * (1.0f / (LN + 1)), x = lo32 + h * (sub + 1);
+      if (hi32 - lo32 <= 4.0f * FLT_EPSILON * tn32 || lo32 + h <= lo32) break;
+      const bool above = x >= hi32 || (x > lo32 && sturm_count32(d32, e232, b0, b1, x) > idx);
+      const unsigned ab = __ballot_sync(gmask, above) & gmask;
+      const int k = ab ? __ffs(ab) - 1 - lane0 : LN;  // the lowest point with more than idx below it
+      const float xk = lo32 + h * (k + 1), xk1 = lo32 + h * k;
+      if (k < LN) hi32 = fminf(hi32, xk);
+      if (k > 0) lo32 = xk1;
+    }
+    const double eps = DBL_EPSILON * 0.5, margin = 8.0 * (double)FLT_EPSILON * T.tnorm;
+    double lo = fmax((double)lo32 - margin, T.gl), hi = fmin((double)hi32 + margin, T.gu);
+    const int c = sturm64_count(d, e2, b0, b1, sub & 1 ? hi : lo, T.tnorm);
+    const int clo = __shfl_sync(gmask, c, lane0), chi = __shfl_sync(gmask, c, lane0 + 1);
+    if (!(clo <= idx && idx < chi)) {
+      lo = T.gl;
+      hi = T.gu;
+    }
+    for (int it = 0; it < 128; ++it) {
+      const double mid = 0.5 * (lo + hi);
+      const double tol = fmax(2.0 * eps * fmax(fabs(lo), fabs(hi)), eps * T.tnorm);
+      if (hi - lo <= tol || mid <= lo || mid >= hi) break;
+      const double h = (hi - lo) / (LN + 1), x = lo + h * (sub + 1);
+      const bool above = (x > lo && x < hi) ? sturm64_count(d, e2, b0, b1, x, T.tnorm) > idx : x >= hi;
+      const unsigned ab = __ballot_sync(gmask, above) & gmask;
+      const int k = ab ? __ffs(ab) - 1 - lane0 : LN;
+      const double xk = lo + h * (k + 1), xk1 = lo + h * k;
+      if (k < LN) hi = fmin(hi, xk);
+      if (k > 0) lo = xk1;
+    }
+    lam = 0.5 * (lo + hi);
+  }
+  if (sub == 0) wslot[(size_t)p * n + j] = lam;
 }
 
 // ---------------------------------------------------------------- kernel 2: eigenvectors
@@ -1172,35 +1266,62 @@ size_t stein_scratch_doubles(int n, int nprob) {
          ((size_t)n * nprob + 1) / 2 + 1 + nprob + 2;
 }
 
+// lanes per eigenvalue of stebz_multi_kernel: as many as leave each warp a scheduler of its own (4
+// per SM), 16 at most; 1: kernels 1 and 1b
+static int stebz_lanes(int n, int nprob) {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    cudaGetLastError();
+    return 1;
+  }
+  int ln = 16;
+  while (ln > 2 && (size_t)n * nprob * ln > (size_t)sms * 4 * 32) ln /= 2;
+  return ln > 2 ? ln : 1;  // (two lanes were slower: n = 211, 24 problems 1.75 ms against 1.37)
+}
+
+int stein_launches(int n, int nprob, int mrrr) { return (mrrr ? 5 : 4) - (stebz_lanes(n, nprob) > 1 ? 1 : 0); }
+
 cudaError_t launch_stein(int n, int nprob, const int32_t* size, const double* d, const double* e, long long strideV,
                          double* w, double* Z, int ld, long long strideZ, double* scratch, int32_t* status,
                          const int32_t* nvec, int nvec_max, int maxits, int mrrr, cudaStream_t st, int* ns2) {
   double* wslot = scratch + (size_t)NARR * n * n * nprob;
   const size_t smem1 = sizeof(double) * 3 * (size_t)n + sizeof(float) * 2 * (size_t)n + sizeof(int) * 2 * (size_t)n;
-  cudaError_t err = cudaFuncSetAttribute(stebz_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1);
-  if (err != cudaSuccess) return err;
-  // the bisection queue (all problems) and the split e^2 live in the inverse-iteration
-  // scratch, unused until kernel 2
+  cudaError_t err = cudaSuccess;
   const size_t cap = (size_t)n * nprob;
-  double* qlo = scratch;
-  double* qhi = qlo + cap;
-  int4* qent = (int4*)(qhi + cap);
-  double* e2g = (double*)(qent + cap);
-  double* tng = e2g + cap;                                            // 5 cap + nprob <= NARR n^2 nprob
-  int* qcount = (int*)(scratch + stein_scratch_doubles(n, nprob) - 2);  // the pad at the end
-  err = cudaMemsetAsync(qcount, 0, sizeof(int), st);
-  if (err != cudaSuccess) return err;
-  dim3 grid1((n + SZ_THREADS - 1) / SZ_THREADS, nprob);
-  stebz_kernel<<<grid1, SZ_THREADS, smem1, st>>>(n, size, d, e, strideV, wslot, status, qcount, qent, qlo, qhi, e2g,
-                                                 tng);
-  err = cudaGetLastError();
-  if (err != cudaSuccess) return err;
-  stebz_bisect_kernel<<<(unsigned)((cap * BQ_LANES + SZ_THREADS - 1) / SZ_THREADS), SZ_THREADS, 0, st>>>(n, d, strideV, e2g, tng,
-                                                                                             wslot, qcount, qent, qlo,
-                                                                                             qhi);
+  const int ln = stebz_lanes(n, nprob);
+  if (ln > 1) {
+    auto fn = ln == 16 ? stebz_multi_kernel<16> : ln == 8 ? stebz_multi_kernel<8> : stebz_multi_kernel<4>;
+    err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1);
+    if (err != cudaSuccess) return err;
+    fn<<<dim3((unsigned)((n * ln + SM_THREADS - 1) / SM_THREADS), nprob), SM_THREADS, smem1, st>>>(n, size, d, e, strideV,
+                                                                                               wslot, status);
+    err = cudaGetLastError();
+    if (err != cudaSuccess) return err;
+  } else {
+    err = cudaFuncSetAttribute(stebz_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1);
+    if (err != cudaSuccess) return err;
+    // the bisection queue (all problems) and the split e^2 live in the inverse-iteration
+    // scratch, unused until kernel 2
+    double* qlo = scratch;
+    double* qhi = qlo + cap;
+    int4* qent = (int4*)(qhi + cap);
+    double* e2g = (double*)(qent + cap);
+    double* tng = e2g + cap;                                            // 5 cap + nprob <= NARR n^2 nprob
+    int* qcount = (int*)(scratch + stein_scratch_doubles(n, nprob) - 2);  // the pad at the end
+    err = cudaMemsetAsync(qcount, 0, sizeof(int), st);
+    if (err != cudaSuccess) return err;
+    dim3 grid1((n + SZ_THREADS - 1) / SZ_THREADS, nprob);
+    stebz_kernel<<<grid1, SZ_THREADS, smem1, st>>>(n, size, d, e, strideV, wslot, status, qcount, qent, qlo, qhi, e2g,
+                                                   tng);
+    err = cudaGetLastError();
+    if (err != cudaSuccess) return err;
+    stebz_bisect_kernel<<<(unsigned)((cap * BQ_LANES + SZ_THREADS - 1) / SZ_THREADS), SZ_THREADS, 0, st>>>(n, d, strideV, e2g, tng,
+                                                                                               wslot, qcount, qent, qlo,
+                                                                                               qhi);
+    err = cudaGetLastError();
+    if (err != cudaSuccess) return err;
+  }
   dim3 grid((n + ST_THREADS - 1) / ST_THREADS, nprob);
-  err = cudaGetLastError();
-  if (err != cudaSuccess) return err;
   int* biglist = (int*)(wslot + (size_t)n * nprob);
   const int bigcap = big_capacity(n, nprob);
   err = cudaMemsetAsync(biglist, 0, sizeof(int), st);
@@ -1235,12 +1356,12 @@ cudaError_t launch_stein(int n, int nprob, const int32_t* size, const double* d,
   err = cudaGetLastError();
   if (err != cudaSuccess) return err;
   // kernel 3: a grid that stays resident; blocks without a listed cluster exit at once
-  const size_t smem3 = sizeof(double) * 5 * (size_t)n + sizeof(int) * 4 * (size_t)n;
-  err = cudaFuncSetAttribute(stein_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem3);
-  if (err != cudaSuccess) return err;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const size_t smem3 = sizeof(double) * 5 * (size_t)n + sizeof(int) * 4 * (size_t)n;
+  err = cudaFuncSetAttribute(stein_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem3);
+  if (err != cudaSuccess) return err;
   stein_cluster_kernel<<<sms, SC_THREADS, smem3, st>>>(n, size, d, e, strideV, wslot, Z, ld, strideZ, scratch, status,
                                                        biglist, bigcap, nvec, nvec_max, maxits, mdone, tgs);
   return cudaGetLastError();
