@@ -31,14 +31,19 @@
 //    FP64 they took as long as the product (an FP64 warp instruction holds its scheduler's
 //    pipe for 64 cycles, and every reduction step is one);
 //  * each warp streams its digits through a ring in shared memory by asynchronous copies;
-//  * global stores wait until the barrier has passed, helpers are not inlined (the kernel has
-//    to stay in the instruction cache), and a reflector's root and reciprocals are Newton steps.
-// A column is now bound by its chain of short phases (~11 us at n = 64), with one block per
+//  * global stores wait until the barrier has passed, and a reflector's root and reciprocals are
+//    Newton steps;
+//  * the kernel is kept small, since a column runs through all of it once: helpers are not
+//    inlined, the product loop takes its plane half at run time and the loops that run once or
+//    twice are not unrolled (108 KB -> 89 KB of code: stage `hetrd` of n = 305, 27 problems
+//    5.8 -> 4.6 ms; peers' shared memory by 32-bit addresses, 77 KB: no faster; the product's units
+//    taken by all 16 warps from a shared counter, 114 KB: 6.9 ms).
+// A column is now bound by its chain of short phases (~7 us at n = 305), with one block per
 // matrix by the stream of digits (16 B per entry and column: at n = 568, 128 problems, the
 // first columns run at 78 % of the measured HBM rate).
-// Measured (stage `hetrd` per step, ms, before -> now): n = 64, 4 problems 3.45 -> 1.52; n = 129,
-// 12 problems 7.8 -> 3.4; n = 305, 27 problems 24.8 -> 11.4; n = 449, 40 problems 39.8 -> 24.7; n = 568,
-// 2 problems 52 -> 23.6; 128 problems 79.3 -> 70.2; n = 2000, 1 problem 458 -> 197.
+// Measured (stage `hetrd` per step, ms, the FP64 panel's products -> now): n = 305, 27 problems
+// 24.8 -> 4.6; n = 449, 40 problems 39.8 -> 10.6; n = 568, 2 problems 52 -> 9.9; 128 problems
+// 79.3 -> 36.2; n = 2000, 1 problem 458 -> 89.
 #include <cooperative_groups.h>
 #include <cuda_fp16.h>
 
@@ -54,8 +59,8 @@ constexpr int HP_MMA_WARPS = 8;                 // warps forming the digit produ
 constexpr int HP_FP_WARPS = HP_THREADS / 32 - HP_MMA_WARPS;
 constexpr int HP_FP_THREADS = 32 * HP_FP_WARPS;
 constexpr int HP_CHUNK = 32;                    // K steps (of 16 columns) of one exact FP32 sum
-constexpr int HP_SLOTS = 16;                    // partial sums of the MMA warps' units
-constexpr int HP_SLOTS2 = 24;                   // and of the others'
+constexpr int HP_SLOTS = 16;                    // partial sums of the product's units
+constexpr int HP_SLOTS2 = 24;                   // and of the panel's products
 constexpr int HP_RED_WARPS = 4;
 constexpr int NB = NAO_HT_NB;
 constexpr int HD_S = 8;                         // digits per value of the FP64 form
@@ -120,7 +125,7 @@ __device__ __forceinline__ double hd_combine(const int* R, int ex) {
 
 // (hi 2^32 + lo) 2^{ex - 56} for |hi| < 2^54, 0 <= lo < 2^54: the two words as orders.  Not inlined:
 // a column runs through the whole kernel once, so the kernel has to fit in the instruction
-// cache (with everything inlined it was 172 KB and every phase waited for instructions).
+// cache (with everything inlined it is 172 KB and every phase waits for instructions).
 __device__ __noinline__ double hd_value(long long hi, long long lo, int ex) {
   const int R[HD_S] = {(int)(hi >> 24), 0, 0, (int)(hi & 0xFFFFFF), (int)(lo >> 24), 0, 0, (int)(lo & 0xFFFFFF)};
   return hd_combine<HD_S>(R, ex);
@@ -241,7 +246,7 @@ __device__ __forceinline__ void hp_copy(uint4* dst, const uint4* src) {
                  :: "r"((uint32_t)__cvta_generic_to_shared(dst + q * 32)), "l"(src + q * 32) : "memory");
 }
 
-// Digit products of plane half H of one 16-row tile over the K steps [k0, k1), added to
+// Digit products of plane half H (0 or 1) of one 16-row tile over the K steps [k0, k1), added to
 // (hi, lo)[4] (row g real, row g imaginary, row g + 8 real, imaginary) in units of 2^{-24} and
 // 2^{-56}; per-lane partial sums (the caller adds the four lanes of a row).  K step k: the A
 // digits at tile + k ts (S x 512 bytes), the B planes' 16 columns at bp + k bs (two parts of
@@ -249,9 +254,9 @@ __device__ __forceinline__ void hp_copy(uint4* dst, const uint4* src) {
 // D > 0: every lane streams its own part of the A digits through a ring of D stages in shared
 // memory (asynchronous copies, 2 KB per stage and warp, so that D K steps are in flight; a lane
 // reads only what it copied itself, so no barrier is needed); D = 0: loads one step ahead.
-template <int S, int H, int D>
+template <int S, int D>
 __device__ __forceinline__ void hp_tile_half(const uint4* tile, int ts, uint4* ring, const __half* bp, int bs, int PS,
-                                             int k0, int k1, int lane, long long* hi, long long* lo) {
+                                             int k0, int k1, int H, int lane, long long* hi, long long* lo) {
   constexpr int SH = S / 2;  // planes of this half; also its uint4 per lane and K step
   const int g = lane >> 2, t = lane & 3;
   const __half* bre = bp + (size_t)g * PS + 4 * t;
@@ -353,8 +358,8 @@ template <int S, int D>
 __device__ __noinline__ longlong2 hp_unit(const uint4* tile, int ts, uint4* ring, const __half* bp, int bs, int PS,
                                              int k0, int k1, int h0, int h1, int lane) {
   long long hi[4] = {0, 0, 0, 0}, lo[4] = {0, 0, 0, 0};
-  if (h0 == 0) hp_tile_half<S, 0, D>(tile, ts, ring, bp, bs, PS, k0, k1, lane, hi, lo);
-  if (h1 == 2) hp_tile_half<S, 1, D>(tile, ts, ring, bp, bs, PS, k0, k1, lane, hi, lo);
+#pragma unroll 1
+  for (int h = h0; h < h1; ++h) hp_tile_half<S, D>(tile, ts, ring, bp, bs, PS, k0, k1, h, lane, hi, lo);
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
     hi[c] = add_quad(hi[c]);
@@ -363,6 +368,24 @@ __device__ __noinline__ longlong2 hp_unit(const uint4* tile, int ts, uint4* ring
   const int tq = lane & 3;
   return make_longlong2(tq == 0 ? hi[0] : tq == 1 ? hi[1] : tq == 2 ? hi[2] : hi[3],
                         tq == 0 ? lo[0] : tq == 1 ? lo[1] : tq == 2 ? lo[2] : lo[3]);
+}
+
+// Global copies of panel column jj (own rows): V below the subdiagonal of A's column (Procedure 3)
+// and the rows of VWr.  They are written while the next column is under way: a cluster barrier
+// with stores to global memory outstanding takes ~4000 cycles instead of ~500.
+__device__ __noinline__ void store_column(z64* __restrict__ Acol, z64* __restrict__ VWrow, const z64* v, const z64* wown,
+                                          int jj, double beta, int C, int rank, int Rown, int Lp, int t0, int nt) {
+#pragma unroll 1
+  for (int lr = t0; lr < Rown; lr += nt) {
+    const int r = ((lr >> 4) * C + rank) * 16 + (lr & 15);
+    if (r < jj || r >= Lp) continue;
+    const z64 vr = v[lr], wr = wown[lr];
+    Acol[r] = r == jj ? zmk(beta, 0.0) : vr;
+    z64* o = VWrow + (size_t)r * 3 * NB + jj;
+    o[0] = vr;
+    o[2 * NB] = vr;
+    o[NB] = wr;
+  }
 }
 
 // sum of `per` slots, 32 apart
@@ -521,23 +544,6 @@ hetrd_panel_mma_kernel(int n, const int32_t* __restrict__ size, z64* __restrict_
   if (tid < 2) s_cx[tid] = 0;
   csync();  // (the other blocks' shared memory exists from here on)
 
-  // global copies of panel column jj (own rows): V below the subdiagonal of A's column
-  // (Procedure 3) and the rows of VWr.  They are written while the next column is under way: a
-  // cluster barrier with stores to global memory outstanding takes ~4000 cycles instead of ~500
-  auto store_column = [&](int jj, double beta, int t0, int nt) {
-#pragma unroll 1
-    for (int lr = t0; lr < Rown; lr += nt) {
-      const int r = row_of(lr);
-      if (r < jj || r >= Lp) continue;
-      const z64 vr = v[lr], wr = wown[lr];
-      A[(size_t)(i0 + jj) * ld + i0 + 1 + r] = r == jj ? zmk(beta, 0.0) : vr;
-      z64* o = VWr + (size_t)(i0 + 1 + r) * 3 * NB;
-      o[jj] = vr;
-      o[2 * NB + jj] = vr;
-      o[NB + jj] = wr;
-    }
-  };
-
   double beta_prev = 0.0;
   int jlast = -1;  // last column whose global copies are still to be written
 #pragma unroll 1
@@ -567,31 +573,19 @@ hetrd_panel_mma_kernel(int n, const int32_t* __restrict__ size, z64* __restrict_
       if (lane == 0) red[wid] = s;
     } else if (j > 0) {
       const int jj = j - 1;
-      // one (four rows, V or W, part) per item
 #pragma unroll 1
-      for (int it = tid - 32 * HP_RED_WARPS; it < 16 * nown; it += HP_THREADS - 32 * HP_RED_WARPS) {
-        const int part = it & 1, vw = (it >> 1) & 1, t = (it >> 2) & 3, lt = it >> 4, c = 2 * jj + vw;
-        const int ex = vw ? s_wx[jj] : 1;
-        const z64* src = (vw ? wown : v) + 16 * lt + 4 * t;
-        unsigned long long z[4], zc[4];
-        const int to = lt * HP_MDT + (c >> 4) * HP_TILE;
-        unsigned char* b1 = hp_base(md1 + to, c & 15, t, part);
-        unsigned char* b2 = hp_base(md2 + to, 4 * t, (c & 15) >> 2, part) + (c & 3);  // row 4 t + l: 64 l on
-#pragma unroll
-        for (int l = 0; l < 4; ++l) {
-          const int r = row_of(16 * lt + 4 * t + l);
-          const double val = (r >= jj && r < Lp) ? (part ? src[l].y : src[l].x) : 0.0;
-          const long long fx = hd_fixed<8>(val, ex);
-          z[l] = hd_bytes<8>(fx);
-          zc[l] = part ? hd_bytes<8>(-fx) : z[l];  // md1 holds conj(M)
-        }
+      for (int it = tid - 32 * HP_RED_WARPS; it < 4 * Rown; it += HP_THREADS - 32 * HP_RED_WARPS) {
+        const int part = it & 1, vw = (it >> 1) & 1, lr = it >> 2, r = row_of(lr), c = 2 * jj + vw, row = lr & 15;
+        const double val = (r >= jj && r < Lp) ? ((const double*)((vw ? wown : v) + lr))[part] : 0.0;
+        const long long fx = hd_fixed<8>(val, vw ? s_wx[jj] : 1);
+        const unsigned long long z = hd_bytes<8>(fx), zc = part ? hd_bytes<8>(-fx) : z;  // md1 holds conj(M)
+        const int to = (lr >> 4) * HP_MDT + (c >> 4) * HP_TILE;
+        unsigned char* b1 = hp_base(md1 + to, c & 15, row >> 2, part) + (row & 3);
+        unsigned char* b2 = hp_base(md2 + to, row, (c & 15) >> 2, part) + (c & 3);
 #pragma unroll
         for (int s = 0; s < 8; ++s) {
-          const int sh = s < 4 ? 32 : 0;
-          *(uint32_t*)(b1 + hp_plane(s)) = gather4((unsigned int)(zc[0] >> sh), (unsigned int)(zc[1] >> sh),
-                                                   (unsigned int)(zc[2] >> sh), (unsigned int)(zc[3] >> sh), 3 - (s & 3));
-#pragma unroll
-          for (int l = 0; l < 4; ++l) b2[64 * l + hp_plane(s)] = (unsigned char)hd_byte<8>(z[l], s);
+          b1[hp_plane(s)] = (unsigned char)hd_byte<8>(zc, s);
+          b2[hp_plane(s)] = (unsigned char)hd_byte<8>(z, s);
         }
       }
     }
@@ -618,7 +612,8 @@ hetrd_panel_mma_kernel(int n, const int32_t* __restrict__ size, z64* __restrict_
         s_cx[1] = 0;
       }
     } else if (j > 0 && wid >= HP_RED_WARPS) {
-      store_column(j - 1, beta_prev, tid - 32 * HP_RED_WARPS, HP_THREADS - 32 * HP_RED_WARPS);
+      store_column(A + (size_t)(i - 1) * ld + i0 + 1, VWr + (size_t)(i0 + 1) * 3 * NB, v, wown, j - 1, beta_prev, C, rank, Rown,
+                   Lp, tid - 32 * HP_RED_WARPS, HP_THREADS - 32 * HP_RED_WARPS);
     }
     __syncthreads();
     const z64 t = s_tau, scale = s_scale;
@@ -654,45 +649,29 @@ hetrd_panel_mma_kernel(int n, const int32_t* __restrict__ size, z64* __restrict_
     longlong2* sl = slots + HP_SLOTS * 32;
     auto fsync = [] { asm volatile("bar.sync 1, %0;" :: "n"(HP_FP_THREADS) : "memory"); };
 
-    if (wid < HP_MMA_WARPS) {
-      // ---- Procedure 4: p = A22 v of the own rows, from the digits
-      double dacc = 0.0;  // this lane's part of Re(p^H v)
-      if (active && nl > 0) {
-        const int nk = NT - ks0;
-        const bool whole = nl >= HP_MMA_WARPS;  // a tile per unit, else (tile, K segment, plane half)
-        int segs = 1, best = 1 << 30;
-        if (!whole)
+    // ---- Procedure 4: p = A22 v of the own rows, from the digits; a tile per unit, or with
+    // few tiles (tile, K segment, plane half)
+    const int nk = NT - ks0;
+    const bool tiles = nl >= HP_MMA_WARPS;
+    int lsegs = 0;
+    if (!tiles) {
+      int best = 1 << 30;
 #pragma unroll 1
-          for (int q = 1; 2 * q * nl <= HP_SLOTS && q <= nk; ++q) {
-            const int cost = (2 * q * nl + HP_MMA_WARPS - 1) / HP_MMA_WARPS * ((nk + q - 1) / q + 4);
-            if (cost < best) best = cost, segs = q;
-          }
-        const int per = whole ? 1 : 2 * segs;
-        auto finish = [&](int lt, longlong2 h) {
-          const int r = 16 * (lt * C + rank) + urow;
-          if (r < j || r >= Lp) return;
-          const double pv = hd_value(h.x, h.y, erow[r] + 1 - 12);
-          ((double*)&pown[16 * lt + urow])[upart] = pv;
-          dacc = fma(pv, ((const double*)&v[16 * lt + urow])[upart], dacc);
-        };
-#pragma unroll 1
-        for (int u = wid; u < nl * per; u += HP_MMA_WARPS) {
-          const int lt = lt0 + u / per, w = u % per, sg = whole ? 0 : w >> 1;
-          const longlong2 h = hp_unit<S, D>(digp + (size_t)(lt * C + rank) * NTn * S * 32, S * 32, ring, vd, 16, PS,
-                                            ks0 + sg * nk / segs, ks0 + (sg + 1) * nk / segs, whole ? 0 : w & 1,
-                                            whole ? 2 : (w & 1) + 1, lane);
-          if (whole) finish(lt, h);
-          else slots[u * 32 + lane] = h;
-        }
-        if (!whole) {
-          asm volatile("bar.sync 2, %0;" :: "n"(32 * HP_MMA_WARPS) : "memory");
-#pragma unroll 1
-          for (int q = wid; q < nl; q += HP_MMA_WARPS) finish(lt0 + q, hp_sum(slots + q * per * 32 + lane, per));
-        }
+      for (int q = 0; (2 * nl << q) <= HP_SLOTS && (1 << q) <= nk; ++q) {
+        const int cost = ((2 * nl << q) + HP_MMA_WARPS - 1) / HP_MMA_WARPS * ((nk >> q) + 5);
+        if (cost < best) best = cost, lsegs = q;
       }
-      dacc = warp_sum(dacc);
-      if (lane == 0) aw[wid] = dacc;
-    } else {
+    }
+    const int lper = tiles ? 0 : lsegs + 1;  // log2 of the units per tile
+    double dacc = 0.0;  // this lane's part of Re(p^H v)
+    auto finish = [&](int lt, longlong2 h) {
+      const int r = 16 * (lt * C + rank) + urow;
+      if (r < j || r >= Lp) return;
+      const double pv = hd_value(h.x, h.y, erow[r] + 1 - 12);
+      ((double*)&pown[16 * lt + urow])[upart] = pv;
+      dacc = fma(pv, ((const double*)&v[16 * lt + urow])[upart], dacc);
+    };
+    if (wid >= HP_MMA_WARPS) {
       // ---- the panel's products
       const int fw = wid - HP_MMA_WARPS;
       if (more && fw == HP_FP_WARPS - 1 && j + 1 < Lp && rank == ((j + 1) >> 4) - C * div_c((j + 1) >> 4)) {
@@ -749,6 +728,26 @@ hetrd_panel_mma_kernel(int n, const int32_t* __restrict__ size, z64* __restrict_
           }
         }
       }
+    }
+    if (wid < HP_MMA_WARPS) {
+      if (active) {
+#pragma unroll 1
+        for (int u = wid; u < nl << lper; u += HP_MMA_WARPS) {
+          const int lt = lt0 + (u >> lper), w = u - ((u >> lper) << lper), sg = w >> 1;
+          const longlong2 h =
+              hp_unit<S, D>(digp + (size_t)(lt * C + rank) * NTn * S * 32, S * 32, ring, vd, 16, PS, ks0 + (sg * nk >> lsegs),
+                            ks0 + ((sg + 1) * nk >> lsegs), tiles ? 0 : w & 1, tiles ? 2 : (w & 1) + 1, lane);
+          if (tiles) finish(lt, h);
+          else slots[u * 32 + lane] = h;
+        }
+        if (!tiles) {
+          asm volatile("bar.sync 2, %0;" :: "n"(32 * HP_MMA_WARPS) : "memory");
+#pragma unroll 1
+          for (int q = wid; q < nl; q += HP_MMA_WARPS) finish(lt0 + q, hp_sum(slots + (q << lper) * 32 + lane, 1 << lper));
+        }
+      }
+      dacc = warp_sum(dacc);
+      if (lane == 0) aw[wid] = dacc;
     }
     if (C > 1) cluster.sync();  // B2: partial sums ready
     // y = M^H v of all blocks summed (fixed order) and what follows from it: Re(y1^H y2), the
@@ -907,7 +906,9 @@ hetrd_panel_mma_kernel(int n, const int32_t* __restrict__ size, z64* __restrict_
         for (int k = 0; k < C; ++k) cluster.map_shared_rank(cfn, k)[c ^ 1] = zconj(crow[c]);
     csync();  // B1: column i + 1 is in every block's shared memory
   }
-  if (jlast >= 0) store_column(jlast, beta_prev, tid, HP_THREADS);  // the last column's global copies
+  if (jlast >= 0)  // the last column's global copies
+    store_column(A + (size_t)(i0 + jlast) * ld + i0 + 1, VWr + (size_t)(i0 + 1) * 3 * NB, v, wown, jlast, beta_prev, C, rank,
+                 Rown, Lp, tid, HP_THREADS);
 }
 
 int smem_optin() {
