@@ -972,14 +972,17 @@ int nao_gen_eig_sized(nao_ctx* ctx, int n, int nprob, const nao_c128* H, const n
       int32_t *mP, *nbP, *stH, *nc2;
       void *ozws, *digp, *mdp;
       int *erowp, *ns2;
+      const int32_t* full;  // per X: 0 where it is upper triangular (null: nowhere)
     };
     auto hp_half = [&](int np, cudaStream_t st, const HpHalf& h, cudaEvent_t part3_done) -> int {
       NAO_STAGE("herm_fill", 1, launch_herm_fill(n, np, h.H, snn, nullptr, h.Hf, n, snn, st));
       {
-        GemmDims d{n, n, n, nullptr, h.mP, nullptr};  // Y = Hf X : n x m
+        // Y = Hf X : n x m
+        const GemmDims d{n, n, n, nullptr, h.mP, nullptr, 0, 0, nullptr, NAO_TRI_B, h.full, h.xmap};
         NAO_CUDA_TRY(ctx, run_zgemm(ctx, "zgemm_HX", np, d, 1.0, GemmOperand{h.Hf, snn, 1, n, 0, nullptr},
                                     GemmOperand{h.X, snn, 1, n, 0, h.xmap}, 0.0, h.Y, snn, 1, n, h.ozws, st, dig));
-        GemmDims d2{n, n, n, h.mP, h.mP, nullptr, 1};  // Hp = X^H Y : m x m, lower triangle
+        // Hp = X^H Y : m x m, lower triangle
+        const GemmDims d2{n, n, n, h.mP, h.mP, nullptr, 1, 0, nullptr, NAO_TRI_AH, h.full, h.xmap};
         NAO_CUDA_TRY(ctx, run_zgemm(ctx, "zgemm_XHY", np, d2, 1.0, GemmOperand{h.X, snn, n, 1, 1, h.xmap},
                                     GemmOperand{h.Y, snn, 1, n, 0, nullptr}, 0.0, h.Hp, snn, 1, n, h.ozws, st, dig));
       }
@@ -1002,7 +1005,8 @@ int nao_gen_eig_sized(nao_ctx* ctx, int n, int nprob, const nao_c128* H, const n
         NAO_CUDA_TRY(ctx, e);
         NAO_CUDA_TRY(ctx, backtransform_blocked(ctx, n, np, h.mP, h.nbP, h.Hp, h.tauH, Zh, h.wH, 0, h.V, h.Vf, h.tauc,
                                                 h.Gw, h.Tw, h.Ww, h.VTw, h.ozws, st, dig, 1));
-        GemmDims dc{n, nb, n, nullptr, h.nbP, h.mP};  // C = X V(:, :nb) : n x nb, row-major [n][nb]
+        // C = X V(:, :nb) : n x nb, row-major [n][nb]
+        const GemmDims dc{n, nb, n, nullptr, h.nbP, h.mP, 0, 0, nullptr, NAO_TRI_A, h.full, h.xmap};
         NAO_CUDA_TRY(ctx, run_zgemm(ctx, "zgemm_XV", np, dc, 1.0, GemmOperand{h.X, snn, 1, n, 0, h.xmap},
                                     GemmOperand{h.V, snn, 1, n, 0, nullptr}, 0.0, h.C, (long long)n * nb, nb, 1,
                                     h.ozws, st, dig));
@@ -1024,6 +1028,7 @@ int nao_gen_eig_sized(nao_ctx* ctx, int n, int nprob, const nao_c128* H, const n
       h.H = (const z64*)H + (size_t)p0 * nn;
       h.X = s_of_prob ? X : X + (size_t)p0 * nn;
       h.xmap = s_of_prob ? s_of_prob + p0 : nullptr;
+      h.full = on && !s_of_prob ? on + p0 : on;
       h.Hf = Hf + (size_t)p0 * nn;
       h.Y = Y + (size_t)p0 * nn;
       h.Hp = Hp + (size_t)p0 * nn;
@@ -1074,10 +1079,12 @@ int nao_gen_eig_sized(nao_ctx* ctx, int n, int nprob, const nao_c128* H, const n
   // ---- Part 3: H' = X^H H X
   NAO_STAGE("herm_fill", 1, launch_herm_fill(n, nprob, (const z64*)H, snn, nullptr, Hf, n, snn, st));
   {
-    GemmDims d{n, n, n, nullptr, mP, nullptr};  // Y = Hf X : n x m
+    // Y = Hf X : n x m
+    const GemmDims d{n, n, n, nullptr, mP, nullptr, 0, 0, nullptr, NAO_TRI_B, on, s_of_prob};
     NAO_CUDA_TRY(ctx, run_zgemm(ctx, "zgemm_HX", nprob, d, 1.0, GemmOperand{Hf, snn, 1, n, 0, nullptr},
                                 GemmOperand{X, snn, 1, n, 0, s_of_prob}, 0.0, Y, snn, 1, n, ozws, st, dig));
-    GemmDims d2{n, n, n, mP, mP, nullptr, 1};  // Hp = X^H Y : m x m, lower triangle
+    // Hp = X^H Y : m x m, lower triangle
+    const GemmDims d2{n, n, n, mP, mP, nullptr, 1, 0, nullptr, NAO_TRI_AH, on, s_of_prob};
     NAO_CUDA_TRY(ctx, run_zgemm(ctx, "zgemm_XHY", nprob, d2, 1.0, GemmOperand{X, snn, n, 1, 1, s_of_prob},
                                 GemmOperand{Y, snn, 1, n, 0, nullptr}, 0.0, Hp, snn, 1, n, ozws, st, dig));
   }
@@ -1160,7 +1167,8 @@ int nao_gen_eig_sized(nao_ctx* ctx, int n, int nprob, const nao_c128* H, const n
     if (C) NAO_STAGE("refine", 1, launch_oa_gather(n, nprob, nb, perm, Cf, n, cfs, (z64*)C, st));
   } else {
     if (C) {
-      GemmDims d{n, nb, n, nullptr, nbP, mP};  // C = X V(:, :nb) : n x nb, row-major [n][nb]
+      // C = X V(:, :nb) : n x nb, row-major [n][nb]
+      const GemmDims d{n, nb, n, nullptr, nbP, mP, 0, 0, nullptr, NAO_TRI_A, on, s_of_prob};
       NAO_CUDA_TRY(ctx, run_zgemm(ctx, "zgemm_XV", nprob, d, 1.0, GemmOperand{X, snn, 1, n, 0, s_of_prob},
                                   GemmOperand{V, snn, 1, n, 0, nullptr}, 0.0, (z64*)C, (long long)n * nb, nb, 1, ozws,
                                   st, dig));

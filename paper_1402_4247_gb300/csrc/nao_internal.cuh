@@ -279,7 +279,11 @@ struct GemmDims {
   int k0 = 0;                           // contraction chunk start: with Kp, problem p's length
                                         // is min(max(Kp[p] - k0, 0), K)
   const int32_t* on = nullptr;          // problems with on[p] = 0 are left out (nullable: all)
+  int tri = 0;                          // NAO_TRI_*: which operand is X, upper triangular in the
+  const int32_t* full = nullptr;        // problems p with full[fmap ? fmap[p] : p] = 0 (null: in none);
+  const int32_t* fmap = nullptr;        // the FP64 CUDA-core route multiplies the zeros
 };
+enum { NAO_TRI_B = 1, NAO_TRI_AH = 2, NAO_TRI_A = 3 };  // B = X, A = X^H, A = X
 // per-problem contraction length of a (possibly chunked) product
 __host__ __device__ inline int gemm_k(const GemmDims& d, int p) {
   if (!d.Kp) return d.K;
