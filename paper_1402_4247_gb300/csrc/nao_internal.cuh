@@ -305,15 +305,14 @@ cudaError_t launch_sym_minus_identity(int n, int nprob, const int32_t* ncols, do
 cudaError_t launch_ns_correct(int n, int nprob, const int32_t* size, const int32_t* ncols, const double* Z,
                               const double* G, int ld, long long stride, double* Z2, cudaStream_t st);
 
-// FP64-accurate complex GEMM on the BF16 tensor cores (digit-plane splitting): C = alpha
-// op(A) op(B) + beta C with real alpha, beta.  Contractions longer than 896 (1792 real) run
-// as chunks whose FP32 group sums stay exact, accumulated in FP64.  ws: zgemm_oz_workspace
-// bytes; err: the context's dev_flags (err[NAO_FLAG_TIMEOUT] set to 1 if a bounded wait
-// expired; the bound is the long long at err + NAO_FLAG_WAIT).  digits: base-64 planes per
-// operand: NAO_OZ_DIGITS_FP64 (ten planes, 60 bits: FP64 accuracy, 55 tensor-core products),
-// or 5, 6, 7 (30, 36, 42 bits: 15, 21, 28 products) for terms that tolerate less, or
-// NAO_OZ_DIGITS_B128: nine base-128 planes (63 bits, 45 products in 17 MMAs per K step
-// instead of 27-31), FP64 accuracy for short contractions (chunks of 256, 512 real).
+// FP64-accurate complex GEMM on the tensor cores (digit-plane splitting): C = alpha op(A) op(B)
+// + beta C with real alpha, beta.  Long contractions run as chunks whose FP32 group sums stay
+// exact, accumulated in FP64.  ws: zgemm_oz_workspace bytes; err: the context's dev_flags
+// (err[NAO_FLAG_TIMEOUT] set to 1 if a bounded wait expired; the bound is the long long at err +
+// NAO_FLAG_WAIT).  digits: NAO_OZ_DIGITS_FP64 (FP64 accuracy: nine base-128 bf16 planes, 63 bits, up to
+// 256 terms, 512 real, else twelve base-32 e4m3 planes, 59 bits, in chunks of 1488, 2976 real), or 5, 6, 7
+// base-64 planes (30, 36, 42 bits: 15, 21, 28 products) for terms that tolerate less;
+// NAO_OZ_DIGITS_B128: the nine base-128 planes in any case (chunks of 256, 512 real).
 constexpr int NAO_OZ_DIGITS_FP64 = 10;
 constexpr int NAO_OZ_DIGITS_B128 = 9;
 constexpr int NAO_OZ_DIGITS_NS = 5;   // the Newton-Schulz correction term (~1e-9 of Z)
@@ -324,7 +323,7 @@ cudaError_t launch_zgemm_oz(int nprob, GemmDims dims, double alpha, GemmOperand 
                             long long Cbs, long long Crs, long long Ccs, void* ws, int* err, cudaStream_t st,
                             int digits = NAO_OZ_DIGITS_FP64);
 
-// The same method for real float64 operands (C = alpha op(A) op(B) + beta C, K <= 1792);
+// The same method for real float64 operands (C = alpha op(A) op(B) + beta C);
 // fits in the workspace of a complex product of the same M, N, K.
 bool dgemm_oz_supported(GemmDims dims);
 size_t dgemm_oz_workspace(int nprob, GemmDims dims);  // bytes of ws for launch_dgemm_oz

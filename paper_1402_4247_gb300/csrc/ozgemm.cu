@@ -1,4 +1,4 @@
-// FP64-accurate complex GEMM on the BF16 tensor cores (tcgen05), for the GEMM-shaped steps
+// FP64-accurate complex GEMM on the BF16 and FP8 tensor cores (tcgen05), for the GEMM-shaped steps
 // of the band step (Sec. 3: Parts 3-4 use ZGEMM; the back-transformation and Part 6 are
 // products too).  On this GPU FP64 runs at 1.2 TFLOP/s and BF16 tcgen05 at ~2.4 PFLOP/s, so
 // an exact splitting of the FP64 operands into small-integer digit planes (the error-free
@@ -9,20 +9,29 @@
 //  * complex -> real: C'' = A' B'' with A' = [Re op(A) | Im op(A)] (M x 2K) and the columns
 //    of B'' interleaved, column 2j = (Re b_j ; -Im b_j), 2j+1 = (Im b_j ; Re b_j), so
 //    C''(:, 2j) = Re c_j and C''(:, 2j+1) = Im c_j;
-//  * every row of A' (column of B'') is scaled by a power of two 2^e so that |x| < 2^e, then
-//    q = round(x 2^{60-e}) (int64, exact integer arithmetic on the FP64 bits) is written in
-//    ten signed base-64 digits d_1..d_10 (|d_1| <= 64, |d_s| <= 32): 60 bits, so that even
-//    entries far below their row's maximum keep FP64-level accuracy in the product;
-//  * digit planes are stored as BF16 (exact): A_s = d_s 2^{-6(s-1)}, B_t = d_t 2^{-6(t-6)};
-//  * the 55 products A_s B_t with s + t <= 11 run on tcgen05 (M = 128, N = 64, K = 16,
-//    FP32 accumulation in TMEM).  Products of one "group" g = s + t share a power-of-two
-//    scale, so for g <= 8 their FP32 sums are exact integers while below 2^24 (guaranteed
-//    for 2K <= 1792); these seven groups get one TMEM accumulator each.  Groups 9..11 share an
-//    eighth (8 x 64 columns = all 512 of TMEM): it is 2^-12 below group 7, so the FP32
-//    rounding it collects over thousands of MMAs stays below FP64 rounding of the result
-//    (sharing one accumulator from group 7 or 8 on was measured 2-10x less accurate);
-//  * epilogue: the exact groups are combined in int64 (units of group 8), the sum of
-//    everything converted to FP64 once and scaled by 2^{e_i + f_j - 42}; real alpha, beta.
+//  * every row of A' (column of B'') is scaled by a power of two 2^e so that |x| < 2^e, rounded to a
+//    fixed-point integer (on the FP64 bits) and written in S balanced digits; the products A_s B_t
+//    with s + t < S (0-based) run on tcgen05 (M = 128, FP32 accumulation in TMEM).  Products of one
+//    group s + t share a power of two, so a group's FP32 sums are exact integers while below 2^24,
+//    and one TMEM accumulator per group keeps them;
+//  * three digit forms:
+//      e4m3, base 32, S = 12 (59 bits; e4m3 holds the integers up to 16): FP64 accuracy for more
+//        than 256 terms (512 real); all twelve groups exact to K' = 5461;
+//      bf16, base 128, S = 9 (63 bits, exact to K' = 512): FP64 accuracy for shorter contractions;
+//      bf16, base 64, S = 5, 6, 7 (30 to 42 bits): terms that tolerate less.
+//    bf16 planes carry the digit's weight, A_s = d_s 2^{-b s}, B_t = d_t 2^{30 - b t}; the groups of
+//    base 128 beyond the eighth share its accumulator, 2^-35 below the first group;
+//  * epilogue: the exact groups are combined in int64, the sum converted to FP64 once and scaled
+//    by the rows' and columns' powers of two; real alpha, beta.
+// What bounds it: an MMA with A from shared memory costs max(N / 2, ~48) cycles for K = 16 bf16 or 32
+// e4m3 columns (measured, N = 32 .. 256), so the digit planes t of B are stacked into operands of up
+// to 256 rows; the operands' shared-memory traffic then sets the pace.  A K step of 32 with e4m3
+// digits takes ~2070 cycles per 32 columns (16 MMAs, 60 KB); ten base-64 bf16 planes (55 products in
+// 31 MMAs, as accurate) took 2 x 2820 per 64 and wrote 1.7 times the bytes.  Measured (splits
+// included): 24 products of 301 x 257 x 420 625 -> 450 us; n = 568, 128 problems, H X 7.1 -> 5.5 ms;
+// n = 2000, H X 2.0 -> 1.4.  Contractions of 96 (256) terms with the twelve e4m3 planes instead of the nine
+// base-128 ones, which leave TMEM for two blocks per SM: rank-2k updates of n = 568, 128 problems 11.2
+// against 9.5 ms, density phase sums 7.0 against 5.2: hence the line at 256.
 // Pipeline: the digit tiles of each K step (16) arrive in one of three shared-memory stages
 // by bulk asynchronous copies (TMA) issued by one producer thread; one thread issues the
 // MMAs and commits them to the stage's barrier.  Every wait is bounded (clock64; the
@@ -30,16 +39,18 @@
 // an error, waits for its issued MMAs and lets its issued copies land (both with the fixed
 // long bound), skips its epilogue and still frees its tensor memory.
 #include <cuda_bf16.h>
+#include <cuda_fp16.h>
+#include <cuda_fp8.h>
 
 #include "nao_internal.cuh"
 
 namespace {
 
-constexpr int OZ_S = 10;             // digit planes per operand for FP64 accuracy (60 bits); the most
-                                     // any product uses (the workspace is sized for it)
+constexpr int OZ_WS_PLANES = 10;     // bf16 planes that the workspace holds (12 e4m3 planes take less)
 constexpr int OZ_BM = 128;           // tile rows (C'' rows)
 constexpr int OZ_BN = 64;            // tile columns (C'' columns = 32 complex columns); B plane tile rows
-constexpr int OZ_BK = 16;            // K' per MMA step
+constexpr int OZ_BK = 16;            // K' per MMA step (bf16 digits; 32 with e4m3 digits: the same bytes)
+__host__ __device__ constexpr int oz_bk(int DB) { return DB == 5 ? 2 * OZ_BK : OZ_BK; }
 constexpr int OZ_TILE_A = OZ_BM * OZ_BK * 2;  // bytes of one A plane tile (4096)
 constexpr int OZ_TILE_B = OZ_BN * OZ_BK * 2;  // bytes of one B plane tile (2048)
 constexpr int OZ_STAGES = 3;
@@ -48,6 +59,7 @@ constexpr int OZ_STAGES = 3;
 // the other's MMAs; their B tiles are the contiguous 32-row halves of the 64-row plane tiles.
 constexpr int OZ_SHORT_KSTEPS = 16;
 constexpr int OZ_THREADS = 256;
+__host__ __device__ constexpr int oz_threads(int DB) { return DB == 5 ? 2 * OZ_THREADS : OZ_THREADS; }
 constexpr long long OZ_WAIT_CYCLES = NAO_TC_WAIT_DEFAULT;  // ~2 s at 2 GHz
 constexpr int OZ_MAX_K2 = 1792;      // 2K bound for exact FP32 group sums (group 8: 9 2^10 per k)
 
@@ -64,10 +76,9 @@ __device__ __forceinline__ uint64_t oz_desc(uint32_t saddr) {
 constexpr uint32_t OZ_IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(OZ_BN >> 3) << 17) |
                               ((uint32_t)(OZ_BM >> 4) << 24);
 
-// byte offset of element (row, k) inside a plane tile (rows x 16 K, bf16)
-__device__ __forceinline__ int oz_tile_off(int row, int k) {
-  return (row >> 3) * 256 + ((k >> 3) & 1) * 128 + (row & 7) * 16 + (k & 7) * 2;
-}
+// byte offset of 16-byte chunk `half` (0 or 1) of a row inside a plane tile (rows x one K step: 16
+// bf16 or 32 e4m3)
+__device__ __forceinline__ int oz_tile_off(int row, int half) { return (row >> 3) * 256 + half * 128 + (row & 7) * 16; }
 
 // biased exponent field of x (0 for zero / subnormal)
 __device__ __forceinline__ int exp_field(double x) { return (int)((__double_as_longlong(x) >> 52) & 0x7ff); }
@@ -166,18 +177,61 @@ __device__ __forceinline__ uint32_t oz_bf16_bits(int d, int k) {
   return d ? (__float_as_uint((float)d) >> 16) + (uint32_t)(k << 7) : 0u;
 }
 
-// Contraction range [klo, khi) (multiples of 16, or the end K) of the output tile that starts at row
+// the digits of the entries q(0), q(1), .. of a lane's 16-byte chunk: plane s's chunk in pk[s].
+// bf16 (DB 6 or 7): 8 entries d 2^{scale0 - DB s}.  e4m3 (DB = 5, S = 12): 16 entries d; the balanced digits
+// d + 16 are the 5-bit fields of q + 16 sum_s 32^s (the top one up to 32), taken for two entries
+// at a time from words that hold three fields of each in their halves, as f16 1024 + u - 1040
+template <int S, int DB, class Q>
+__device__ __forceinline__ void oz_pack(uint32_t (&pk)[S][4], int scale0, Q q) {
+  if constexpr (DB == 5) {
+    static_assert(S == 12, "four words of three 5-bit digits");
+#pragma unroll
+    for (int w = 0; w < 4; ++w)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const unsigned long long bias = 0x842108421084210ull;  // 16 in each of the twelve 5-bit fields
+        const unsigned long long z0 = (unsigned long long)q(4 * w + 2 * h) + bias, z1 = (unsigned long long)q(4 * w + 2 * h + 1) + bias;
+#pragma unroll
+        for (int part = 0; part < 4; ++part) {  // digits 3 part .. 3 part + 2
+          const int sh = 45 - 15 * part;
+          const uint32_t keep = part ? 0x7fffu : 0xffffu;
+          const uint32_t y = ((uint32_t)(z0 >> sh) & keep) | ((uint32_t)(z1 >> sh) & keep) << 16;
+#pragma unroll
+          for (int k = 0; k < 3; ++k) {
+            const uint32_t field = part == 0 && k == 0 ? 0x003f003fu : 0x001f001fu;
+            const uint32_t u = ((y >> (10 - 5 * k)) & field) | 0x64006400u;  // 1024 + (d + 16) in f16
+            const __half2 x = __hsub2(*(const __half2*)&u, __half2{__ushort_as_half(0x6410), __ushort_as_half(0x6410)});
+            const uint32_t b = __nv_cvt_halfraw2_to_fp8x2(*(const __half2_raw*)&x, __NV_SATFINITE, __NV_E4M3);
+            pk[3 * part + k][w] = h ? pk[3 * part + k][w] | b << 16 : b;
+          }
+        }
+      }
+  } else {
+#pragma unroll
+    for (int s = 0; s < S; ++s) pk[s][0] = pk[s][1] = pk[s][2] = pk[s][3] = 0u;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      int d[S];
+      oz_digits<S, DB>(q(e), d);
+#pragma unroll
+      for (int s = 0; s < S; ++s) pk[s][e >> 1] |= oz_bf16_bits(d[s], scale0 - DB * s) << (16 * (e & 1));
+    }
+  }
+}
+
+// Contraction range [klo, khi) (multiples of a K step, or the end K) of the output tile that starts at row
 // row0 and ends before column col1, where X is upper triangular (GemmDims::tri): X(k, j) = 0 for
 // k > j.  Outside it the products are exact zeros, so results do not depend on the range.  An
-// empty range (a later chunk of a long contraction) becomes the first 16.
+// empty range (a later chunk of a long contraction) becomes the first step.
 // Half of H X and X V and a third of the lower triangle of X^H Y are such zeros; measured at
 // n = 568, 128 problems (ms, splits included): H X 10.5 -> 7.1, X^H Y 7.2 -> 6.1, X V 10.6 -> 7.1.
+template <int BK>
 __device__ __forceinline__ void oz_krange(const GemmDims& d, int p, int K, int row0, int row1, int col1, int& klo, int& khi) {
   klo = 0, khi = K;
   if (!d.tri || !d.full || d.full[d.fmap ? d.fmap[p] : p]) return;
-  if (d.tri == NAO_TRI_A) klo = min(max(row0 - d.k0, 0), K) & ~15;
-  else khi = min(max(((d.tri == NAO_TRI_B ? col1 : row1) - d.k0 + 15) & ~15, 0), K);
-  if (klo >= khi) klo = 0, khi = min(16, K);
+  if (d.tri == NAO_TRI_A) klo = min(max(row0 - d.k0, 0), K) & ~(BK - 1);
+  else khi = min(max(((d.tri == NAO_TRI_B ? col1 : row1) - d.k0 + BK - 1) & ~(BK - 1), 0), K);
+  if (klo >= khi) klo = 0, khi = min(BK, K);
 }
 
 // K steps of the planes that hold the entries [klo, khi) of both halves of K' (one range when REAL):
@@ -186,16 +240,16 @@ struct OzSteps {
   int a0, a1, b0, b1;
   __device__ bool has(int c) const { return (c >= a0 && c < a1) || (c >= b0 && c < b1); }
 };
-template <bool REAL>
+template <bool REAL, int BK>
 __device__ __forceinline__ OzSteps oz_steps(int K2p, int K, int klo, int khi) {
-  const int nks = K2p / OZ_BK;
+  const int nks = K2p / BK;
   OzSteps s;
-  s.a0 = klo / OZ_BK;
-  s.a1 = min(nks, (khi + OZ_BK - 1) / OZ_BK);
+  s.a0 = klo / BK;
+  s.a1 = min(nks, (khi + BK - 1) / BK);
   s.b0 = s.b1 = s.a1;
   if (!REAL) {
-    s.b0 = (K2p / 2 + klo) / OZ_BK;
-    s.b1 = min(nks, (K2p / 2 + khi + OZ_BK - 1) / OZ_BK);
+    s.b0 = (K2p / 2 + klo) / BK;
+    s.b1 = min(nks, (K2p / 2 + khi + BK - 1) / BK);
     if (s.b0 <= s.a1) s.a1 = s.b0 = s.b1;
   }
   return s;
@@ -207,7 +261,8 @@ __device__ __forceinline__ OzSteps oz_steps(int K2p, int K, int klo, int khi) {
 //   B (IS_B = true):  the rows of B''^T, i.e. the columns of B'' (2N interleaved columns when
 //                     complex: row 2j = (Re b_j ; -Im b_j), row 2j+1 = (Im b_j ; Re b_j)).
 // Plane layout (K-major tiles of TR = 128 (A) or 64 (B) rows x 16 K, bf16):
-//   planes[prob][s][row / TR][k' / 16][oz_tile_off(row % TR, k' % 16)].
+//   planes[prob][s][row / TR][k' / 16][oz_tile_off(row % TR, (k' % 16) / 8) + 2 (k' % 8)];
+// e4m3 planes: 32 and 16 in place of 16 and 8, one byte per entry.
 // Complex operands: K' = 2 Kh with Kh = round_up(K, 8); entries 0..K-1 hold the first
 // part (Re op(A); Re b or Im b), entries Kh..Kh+K-1 the second, the rest are zero, so that
 // both halves start on an 8-entry (16-byte) boundary.
@@ -224,7 +279,9 @@ __global__ void __launch_bounds__(256) oz_split(int nprob, GemmDims dims, GemmOp
                                                  __nv_bfloat16* __restrict__ planes, int* __restrict__ xexp) {
   constexpr int TR = IS_B ? OZ_BN : OZ_BM;            // rows per plane tile
   constexpr int TB = TR * OZ_BK * 2;                  // bytes per plane tile
-  constexpr int SCALE0 = IS_B ? 30 : 0;               // plane s holds d_s 2^{SCALE0 - DB s}
+  constexpr int SCALE0 = IS_B ? 30 : 0;               // plane s holds d_s 2^{SCALE0 - DB s} (e4m3: d_s)
+  constexpr int BK = oz_bk(DB), E = BK / 2;           // K' per step; entries per 16-byte chunk of a plane
+  constexpr int PASS = 8 * BK;                        // entries that the block's warps take at a time
   const int p = blockIdx.y;
   if (dims.on && !dims.on[p]) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -246,9 +303,9 @@ __global__ void __launch_bounds__(256) oz_split(int nprob, GemmDims dims, GemmOp
   // pass 1: largest exponent field over the row's values
   int bmax = 0;
   if (live)
-    for (int k = warp * 16 + kh * 8; k < K; k += 8 * 16) {
+    for (int k = warp * BK + kh * E; k < K; k += PASS) {
 #pragma unroll
-      for (int e = 0; e < 8; ++e) {
+      for (int e = 0; e < E; ++e) {
         if (k + e >= K) break;
         if (REAL) {
           bmax = max(bmax, exp_field(((const double*)xb)[at(k + e)]));
@@ -273,53 +330,47 @@ __global__ void __launch_bounds__(256) oz_split(int nprob, GemmDims dims, GemmOp
       xexp[(size_t)p * Rp + row] = ex;
     }
   }
-  // pass 2: digits of 8 consecutive K' entries per thread, one 16-byte store per plane
+  // pass 2: digits of E consecutive K' entries per thread, one 16-byte store per plane
   const int Kh = REAL ? K2p : K2p / 2;  // start of the second half of K' (complex)
-  const int nks = K2p / OZ_BK;
+  const int nks = K2p / BK;
   // the K range that the products read of this row's plane tile
   int klo = 0, khi = K;
   if (!REAL && (dims.tri == NAO_TRI_B) == IS_B) {
     const int t0 = row / TR * TR;
-    oz_krange(dims, p, K, t0, t0 + TR, (t0 + TR) / 2, klo, khi);
+    oz_krange<BK>(dims, p, K, t0, t0 + TR, (t0 + TR) / 2, klo, khi);
   }
   const size_t plane_bytes = (size_t)(Rp / TR) * nks * TB;
   unsigned char* pl0 = (unsigned char*)planes + (size_t)p * S * plane_bytes;
   if (IS_B && !REAL) {
-    // 8-groups g of the first half: own row at K' = 8 g, the partner row (same complex
-    // column, other part) at K' = Kh + 8 g; both rows lie in the same plane tile
-    const int ng = Kh / 8;
+    // groups g of E entries of the first half: own row at K' = E g, the partner row (same complex
+    // column, other part) at K' = Kh + E g; both rows lie in the same plane tile
+    const int ng = Kh / E;
     const int prow = row ^ 1;
     unsigned char* rb0 = pl0 + (size_t)(row / TR) * nks * TB;
     const bool cj = X.conj != 0;
     // lane h = 0: Re b' = Re b to both rows; h = 1: Im b' = (cj ? -1 : 1) Im b to its own row
     // and its negation to the partner's second half
     const bool neg = h == 1 && cj;
-    const uint32_t pflip = h == 1 ? 0x80008000u : 0u;  // bf16 sign bits (a zero becomes -0)
+    const uint32_t pflip = h == 1 ? (DB == 5 ? 0x80808080u : 0x80008000u) : 0u;  // sign bits (a zero becomes -0)
     const bool cut = khi < K;  // (NAO_TRI_B: klo = 0)
     for (int g = 2 * warp + kh; g < ng; g += 16) {
-      // a K step of the second half may start 8 entries off the first half's and reads one group
+      // a K step of the second half may start one group off the first half's and reads one group
       // more; the last group shares its step with the second half's first
-      if (cut && g > khi / 8 && g < ng - 1) continue;
+      if (cut && g > khi / E && g < ng - 1) continue;
       uint32_t pk[S][4];
-#pragma unroll
-      for (int s2 = 0; s2 < S; ++s2) pk[s2][0] = pk[s2][1] = pk[s2][2] = pk[s2][3] = 0u;
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const int k = 8 * g + e;
+      oz_pack<S, DB>(pk, SCALE0, [&](int e) -> long long {
+        const int k = E * g + e;
         double v = 0.0;
         if (live && k < K) {
           const z64 z = ((const z64*)xb)[at(k)];
           v = h ? z.y : z.x;
         }
-        const long long q = oz_fixed<S, DB>(v, ex);
-        int d[S];
-        oz_digits<S, DB>(neg ? -q : q, d);
-#pragma unroll
-        for (int s2 = 0; s2 < S; ++s2) pk[s2][e >> 1] |= oz_bf16_bits(d[s2], SCALE0 - DB * s2) << (16 * (e & 1));
-      }
+        const long long q = oz_fixed<S, DB>(v, DB == 5 ? ex + 1 : ex);
+        return neg ? -q : q;
+      });
       const int g2 = ng + g;
-      unsigned char* own = rb0 + (size_t)(g >> 1) * TB + oz_tile_off(row % TR, (g & 1) * 8);
-      unsigned char* par = rb0 + (size_t)(g2 >> 1) * TB + oz_tile_off(prow % TR, (g2 & 1) * 8);
+      unsigned char* own = rb0 + (size_t)(g >> 1) * TB + oz_tile_off(row % TR, g & 1);
+      unsigned char* par = rb0 + (size_t)(g2 >> 1) * TB + oz_tile_off(prow % TR, g2 & 1);
 #pragma unroll
       for (int s2 = 0; s2 < S; ++s2) {
         *(uint4*)(own + (size_t)s2 * plane_bytes) = make_uint4(pk[s2][0], pk[s2][1], pk[s2][2], pk[s2][3]);
@@ -329,17 +380,14 @@ __global__ void __launch_bounds__(256) oz_split(int nprob, GemmDims dims, GemmOp
     }
     return;
   }
-  unsigned char* base = pl0 + (size_t)(row / TR) * nks * TB + oz_tile_off(row % TR, kh * 8);
-  const OzSteps steps = oz_steps<REAL>(K2p, K, klo, khi);
+  unsigned char* base = pl0 + (size_t)(row / TR) * nks * TB + oz_tile_off(row % TR, kh);
+  const OzSteps steps = oz_steps<REAL, BK>(K2p, K, klo, khi);
   const bool cut = klo > 0 || khi < K;
   for (int c = warp; c < nks; c += 8) {
     if (cut && !steps.has(c)) continue;
     uint32_t pk[S][4];
-#pragma unroll
-    for (int s = 0; s < S; ++s) pk[s][0] = pk[s][1] = pk[s][2] = pk[s][3] = 0u;
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const int kk = c * OZ_BK + kh * 8 + e;
+    oz_pack<S, DB>(pk, SCALE0, [&](int e) -> long long {
+      const int kk = c * BK + kh * E + e;
       double v = 0.0;
       bool neg = false;  // negations are applied to the exact integer, not as FP64 instructions
       if (REAL) {
@@ -353,12 +401,9 @@ __global__ void __launch_bounds__(256) oz_split(int nprob, GemmDims dims, GemmOp
           neg = hi && X.conj != 0;  // conj: Im z enters with the opposite sign
         }
       }
-      const long long q = oz_fixed<S, DB>(v, ex);
-      int d[S];
-      oz_digits<S, DB>(neg ? -q : q, d);
-#pragma unroll
-      for (int s = 0; s < S; ++s) pk[s][e >> 1] |= oz_bf16_bits(d[s], SCALE0 - DB * s) << (16 * (e & 1));
-    }
+      const long long q = oz_fixed<S, DB>(v, DB == 5 ? ex + 1 : ex);
+      return neg ? -q : q;
+    });
 #pragma unroll
     for (int s = 0; s < S; ++s)
       *(uint4*)(base + (size_t)s * plane_bytes + (size_t)c * TB) = make_uint4(pk[s][0], pk[s][1], pk[s][2], pk[s][3]);
@@ -367,11 +412,20 @@ __global__ void __launch_bounds__(256) oz_split(int nprob, GemmDims dims, GemmOp
 
 // ---------------------------------------------------------------------------- tensor kernel
 // instruction descriptor for N = nn output columns (a multiple of 16, <= 256)
+template <int DB>
 __device__ __forceinline__ uint32_t oz_idesc(int nn) {
-  return (OZ_IDESC & ~(0x3Fu << 17)) | ((uint32_t)(nn >> 3) << 17);
+  constexpr uint32_t base = DB == 5 ? OZ_IDESC & ~((7u << 7) | (7u << 10)) : OZ_IDESC;  // kind::f8f6f4: e4m3 is 0
+  return (base & ~(0x3Fu << 17)) | ((uint32_t)(nn >> 3) << 17);
 }
 
+template <int DB>
 __device__ __forceinline__ void oz_mma(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
+  if (DB == 5) {
+    asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+                 "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n}\n"
+                 :: "r"(dtmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc));
+    return;
+  }
   asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
                "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
                :: "r"(dtmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc));
@@ -416,7 +470,7 @@ __device__ __forceinline__ void oz_bulk_copy(void* dst_smem, const void* src_gme
 //     to the stage's empty barrier, and after the last stage to the "done" barrier;
 //   all 8 warps: wait for "done", then run the epilogue from TMEM.
 template <bool REAL, int S, int DB, int BN, int NST>
-__global__ void __launch_bounds__(OZ_THREADS, BN == OZ_BN ? 1 : 2)
+__global__ void __launch_bounds__(oz_threads(DB), BN == OZ_BN || DB == 5 ? 1 : 2)
 oz_gemm_kernel(int nprob, GemmDims dims, double alpha, double beta, const __nv_bfloat16* __restrict__ Ap,
                const __nv_bfloat16* __restrict__ Bp, const int* __restrict__ rexp, const int* __restrict__ cexp, int Mp,
                int N2p, int K2p, void* __restrict__ Cv, long long Cbs, long long Crs, long long Ccs, int* __restrict__ err) {
@@ -424,15 +478,16 @@ oz_gemm_kernel(int nprob, GemmDims dims, double alpha, double beta, const __nv_b
   // one also every group beyond it (MERGED).  The first NEX accumulators are combined exactly
   // (their FP32 sums are exact integers: DB = 6 while 2K' <= 1792, DB = 7 while K' <= 512);
   // the rest lie at least 2^-35 below the first group and enter rounded.
-  constexpr int NACC = S < 8 ? S : 8;
+  constexpr int BK = oz_bk(DB);
+  constexpr int NACC = DB == 5 || S < 8 ? S : 8;
   constexpr bool MERGED = S > NACC;
-  constexpr int NEX = DB == 7 ? 6 : (MERGED ? NACC - 1 : NACC);
+  constexpr int NEX = DB == 7 ? 6 : NACC;
   constexpr int TMEM_COLS = NACC * BN <= 128 ? 128 : (NACC * BN <= 256 ? 256 : 512);
   constexpr int TILE_B = BN * OZ_BK * 2;              // bytes of one B tile in shared memory
   constexpr int STAGE = S * (OZ_TILE_A + TILE_B);     // bytes per pipeline stage
   constexpr int kUnitExp = DB * (NEX - 1) - 30;       // an accumulator's value in units of the last exact
                                                       // group: v 2^kUnitExp
-  constexpr int kExp = -DB * (NEX + 1);               // the output is t 2^{e_i + f_j + kExp}
+  constexpr int kExp = DB == 5 ? -33 : -DB * (NEX + 1);  // the output is t 2^{e_i + f_j + kExp - sh}
   extern __shared__ __align__(1024) unsigned char oz_smem[];
   __shared__ uint64_t full_bar[NST], empty_bar[NST], done_bar;
   __shared__ uint32_t tbase;
@@ -449,13 +504,13 @@ oz_gemm_kernel(int nprob, GemmDims dims, double alpha, double beta, const __nv_b
   if (rb * OZ_BM >= M || cb * CPT >= N) return;
   if (dims.lower && cb * CPT > rb * OZ_BM + OZ_BM - 1) return;
   unsigned char* stage0 = (unsigned char*)(((uintptr_t)oz_smem + 1023) & ~(uintptr_t)1023);
-  const int nks = K2p / OZ_BK;  // plane layout (all problems)
+  const int nks = K2p / BK;  // plane layout (all problems)
   // this problem's digit planes hold data in the K steps of its contraction range only (one
   // range when the two halves' steps meet, as for K_p = K)
   const int Kprob = gemm_k(dims, p);
   int klo = 0, khi = Kprob;
-  if (!REAL) oz_krange(dims, p, Kprob, rb * OZ_BM, rb * OZ_BM + OZ_BM, (cb + 1) * CPT, klo, khi);
-  const OzSteps steps = oz_steps<REAL>(K2p, Kprob, klo, khi);
+  if (!REAL) oz_krange<BK>(dims, p, Kprob, rb * OZ_BM, rb * OZ_BM + OZ_BM, (cb + 1) * CPT, klo, khi);
+  const OzSteps steps = oz_steps<REAL, BK>(K2p, Kprob, klo, khi);
   const int s1 = steps.a1 - steps.a0;
   const int nks_p = max(1, s1 + (steps.b1 - steps.b0));
   const size_t aplane = (size_t)(Mp / OZ_BM) * nks * (OZ_TILE_A / 2);
@@ -542,14 +597,14 @@ oz_gemm_kernel(int nprob, GemmDims dims, double alpha, double beta, const __nv_b
         for (int t0 = 0; t0 <= tlast; t0 += WMAX) {
           const int w = min(WMAX, tlast - t0 + 1), acc0 = s + t0;
           const uint32_t on = (init_mask >> acc0) & 1u;
-          oz_mma(tmem + acc0 * BN, ad, oz_desc(sb + t0 * TILE_B), oz_idesc(w * BN), on);
+          oz_mma<DB>(tmem + acc0 * BN, ad, oz_desc(sb + t0 * TILE_B), oz_idesc<DB>(w * BN), on);
           init_mask |= ((1u << w) - 1u) << acc0;
         }
         if (MERGED) {
 #pragma unroll
           for (int t = (tlast + 1 > 0 ? tlast + 1 : 0); t < S && s + t <= S - 1; ++t) {
             const uint32_t on = (init_mask >> (NACC - 1)) & 1u;
-            oz_mma(tmem + (NACC - 1) * BN, ad, oz_desc(sb + t * TILE_B), oz_idesc(BN), on);
+            oz_mma<DB>(tmem + (NACC - 1) * BN, ad, oz_desc(sb + t * TILE_B), oz_idesc<DB>(BN), on);
             init_mask |= 1u << (NACC - 1);
           }
         }
@@ -575,11 +630,12 @@ oz_gemm_kernel(int nprob, GemmDims dims, double alpha, double beta, const __nv_b
         oz_wait(&full_bar[ks % NST], (ks / NST) & 1);
     }
   } else {
-    // epilogue: warp w reads TMEM lanes 32 (w % 4) .. +31 (tile rows); warps 0-3 take
-    // complex columns 0..15 of the tile, warps 4-7 columns 16..31.
+    // epilogue: warp w reads TMEM lanes 32 (w % 4) .. +31 (tile rows) and takes the part w / 4 of
+    // the tile's columns
     const int row = 32 * (warp & 3) + lane;
     const int gi = rb * OZ_BM + row;
-    const int half = warp >> 2;
+    const int part = warp >> 2;  // of the tile's columns
+    constexpr int PARTS = oz_threads(DB) / 128, CW = DB == 5 ? 4 : 8;  // C'' columns per round
     const int erow = (gi < M) ? rexp[(size_t)p * Mp + gi] : 0;
     // alpha = +-2^ae goes into the exponent; any other alpha takes one FP64 multiply
     const long long abits = __double_as_longlong(alpha);
@@ -587,25 +643,45 @@ oz_gemm_kernel(int nprob, GemmDims dims, double alpha, double beta, const __nv_b
     const bool amul = (abits & 0xFFFFFFFFFFFFFll) != 0 || afield == 0 || afield == 0x7ff;
     const int ae = amul ? 0 : afield - 1023;
     const bool aneg = !amul && abits < 0;
-    for (int cc = 0; cc < BN / 4; cc += 4) {  // 8 C'' columns per round
-      const int col0 = half * (BN / 2) + 2 * cc;
-      uint32_t v[NACC][8];
+    for (int cc = 0; cc < BN / PARTS; cc += CW) {
+      const int col0 = part * (BN / PARTS) + cc;
+      uint32_t v[NACC][CW];
 #pragma unroll
       for (int a = 0; a < NACC; ++a) {
         const uint32_t taddr = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + a * BN + col0;
-        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                     : "=r"(v[a][0]), "=r"(v[a][1]), "=r"(v[a][2]), "=r"(v[a][3]), "=r"(v[a][4]), "=r"(v[a][5]),
-                       "=r"(v[a][6]), "=r"(v[a][7])
-                     : "r"(taddr));
+        if constexpr (CW == 4)
+          asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                       : "=r"(v[a][0]), "=r"(v[a][1]), "=r"(v[a][2]), "=r"(v[a][3]) : "r"(taddr));
+        else
+          asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                       : "=r"(v[a][0]), "=r"(v[a][1]), "=r"(v[a][2]), "=r"(v[a][3]), "=r"(v[a][4]), "=r"(v[a][5]),
+                         "=r"(v[a][6]), "=r"(v[a][7])
+                       : "r"(taddr));
       }
       asm volatile("tcgen05.wait::ld.sync.aligned;");
       if (gi >= M) continue;
       // every output as one fixed-point integer t (value t 2^{e_i + f_j + kExp - sh}), turned
       // into a double by integer operations: no FP64 instruction unless beta != 0
-      long long t[8];
-      int sh[8];
+      long long t[CW];
+      int sh[CW];
 #pragma unroll
-      for (int c = 0; c < 8; ++c) {
+      for (int c = 0; c < CW; ++c) {
+        if (DB == 5) {
+          // group a counts in units of 2^{-8 - 5 a} and is exact (2^8 a product, 12 in a group, K' <=
+          // 2976: below 2^24): two words of six groups each, in units of 2^-33 and 2^-63
+          // (|.| < 2^50), joined with the low word rounded at least 2^-60 below the result
+          long long hi = 0, lo = 0;
+#pragma unroll
+          for (int a = 0; a < NACC / 2; ++a) {
+            hi += (long long)__float2int_rn(__uint_as_float(v[a][c])) * (1ll << (5 * (NACC / 2 - 1 - a)));
+            lo += (long long)__float2int_rn(__uint_as_float(v[NACC / 2 + a][c])) * (1ll << (5 * (NACC / 2 - 1 - a)));
+          }
+          const unsigned long long ah = hi < 0 ? 0ull - (unsigned long long)hi : (unsigned long long)hi;
+          const int s = min(max(__clzll((long long)ah) - 3, 0), 30);
+          t[c] = (long long)((unsigned long long)hi << s) + (s == 30 ? lo : (lo + (1ll << (29 - s))) >> (30 - s));
+          sh[c] = s;
+          continue;
+        }
         // exact groups a < NEX: G_a = n_a 2^{30 - DB a} with integer n_a;
         // hi = sum_a n_a 2^{DB (NEX - 1 - a)} counts in units of the last exact group
         long long hi = 0;
@@ -633,7 +709,7 @@ oz_gemm_kernel(int nprob, GemmDims dims, double alpha, double beta, const __nv_b
       if (REAL) {
         double* Cp = (double*)Cv + (size_t)p * Cbs;
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
+        for (int c = 0; c < CW; ++c) {
           const int gj = cb * BN + col0 + c;
           if (gj >= N) continue;
           const int ex = erow + cexp[(size_t)p * N2p + gj] + kExp + ae;
@@ -646,8 +722,8 @@ oz_gemm_kernel(int nprob, GemmDims dims, double alpha, double beta, const __nv_b
       } else {
         z64* Cp = (z64*)Cv + (size_t)p * Cbs;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int gj = cb * (BN / 2) + half * (BN / 4) + cc + q;  // complex column
+        for (int q = 0; q < CW / 2; ++q) {
+          const int gj = cb * (BN / 2) + col0 / 2 + q;  // complex column
           if (gj >= N) continue;
           const int ex = erow + cexp[(size_t)p * (N2p / 2) + gj] + kExp + ae;
           z64* cp = Cp + (long long)gi * Crs + (long long)gj * Ccs;
@@ -675,20 +751,21 @@ oz_gemm_kernel(int nprob, GemmDims dims, double alpha, double beta, const __nv_b
 
 inline int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
-// Split both operands into S digit planes of DB bits and run the tensor kernel.  The plane
-// buffers are laid out for OZ_S planes (the workspace size), whatever S is used.  Base-128
+// Split both operands into S digit planes of DB bits and run the tensor kernel.  The bf16
+// planes' buffers are laid out for OZ_WS_PLANES (the workspace size), whatever S is used.  Base-128
 // digits (DB = 7) always take the 32-column tiles: their contractions are at most 32 K steps.
 template <bool REAL, int S, int DB>
 cudaError_t launch_oz(int nprob, GemmDims dims, double alpha, GemmOperand A, GemmOperand B, double beta, void* C,
                       long long Cbs, long long Crs, long long Ccs, void* ws, int* err, cudaStream_t st) {
   if (nprob <= 0 || dims.M <= 0 || dims.N <= 0) return cudaSuccess;
   const int w2 = REAL ? 1 : 2;
-  const int Mp = round_up(dims.M, OZ_BM), N2p = round_up(w2 * dims.N, OZ_BN), K2p = round_up(w2 * dims.K, OZ_BK);
+  const int Mp = round_up(dims.M, OZ_BM), N2p = round_up(w2 * dims.N, OZ_BN), K2p = round_up(w2 * dims.K, oz_bk(DB));
   unsigned char* w = (unsigned char*)ws;
+  constexpr size_t PER = DB == 5 ? S : 2 * OZ_WS_PLANES;  // bytes per entry
   __nv_bfloat16* Apl = (__nv_bfloat16*)w;
-  w += (size_t)nprob * OZ_S * Mp * K2p * 2;
+  w += (size_t)nprob * PER * Mp * K2p;
   __nv_bfloat16* Bpl = (__nv_bfloat16*)w;
-  w += (size_t)nprob * OZ_S * N2p * K2p * 2;
+  w += (size_t)nprob * PER * N2p * K2p;
   int* rexp = (int*)w;
   int* cexp = rexp + (size_t)nprob * Mp;
   oz_split<false, REAL, S, DB><<<dim3(Mp / 16, nprob), 256, 0, st>>>(nprob, dims, A, Mp, K2p, Apl, rexp);
@@ -697,14 +774,14 @@ cudaError_t launch_oz(int nprob, GemmDims dims, double alpha, GemmOperand A, Gem
   oz_split<true, REAL, S, DB><<<dim3(N2p / 16, nprob), 256, 0, st>>>(nprob, dims, B, N2p, K2p, Bpl, cexp);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  if (DB == 7 || K2p / OZ_BK <= OZ_SHORT_KSTEPS) {
-    constexpr int BN = OZ_BN / 2, NST = 2;
+  if (DB != 6 || K2p / OZ_BK <= OZ_SHORT_KSTEPS) {
+    constexpr int BN = OZ_BN / 2, NST = DB == 5 ? 3 : 2;
     const size_t smem = NST * (size_t)S * (OZ_TILE_A + BN * OZ_BK * 2) + 1024;
     e = cudaFuncSetAttribute(oz_gemm_kernel<REAL, S, DB, BN, NST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem);
     if (e != cudaSuccess) return e;
     dim3 grid(N2p / BN, Mp / OZ_BM, nprob);
-    oz_gemm_kernel<REAL, S, DB, BN, NST><<<grid, OZ_THREADS, smem, st>>>(nprob, dims, alpha, beta, Apl, Bpl, rexp,
+    oz_gemm_kernel<REAL, S, DB, BN, NST><<<grid, oz_threads(DB), smem, st>>>(nprob, dims, alpha, beta, Apl, Bpl, rexp,
                                                                          cexp, Mp, N2p, K2p, C, Cbs, Crs, Ccs, err);
     return cudaGetLastError();
   }
@@ -714,7 +791,7 @@ cudaError_t launch_oz(int nprob, GemmDims dims, double alpha, GemmOperand A, Gem
                              (int)smem);
     if (e != cudaSuccess) return e;
     dim3 grid(N2p / OZ_BN, Mp / OZ_BM, nprob);
-    oz_gemm_kernel<REAL, S, DB, OZ_BN, OZ_STAGES><<<grid, OZ_THREADS, smem, st>>>(
+    oz_gemm_kernel<REAL, S, DB, OZ_BN, OZ_STAGES><<<grid, oz_threads(DB), smem, st>>>(
         nprob, dims, alpha, beta, Apl, Bpl, rexp, cexp, Mp, N2p, K2p, C, Cbs, Crs, Ccs, err);
   }
   return cudaGetLastError();
@@ -724,6 +801,7 @@ cudaError_t launch_oz(int nprob, GemmDims dims, double alpha, GemmOperand A, Gem
 // K' <= OZ_MAX_K2 (real); base-128 digits K' <= 512.
 constexpr int OZ_CHUNK_C = OZ_MAX_K2 / 2, OZ_CHUNK_R = OZ_MAX_K2;
 constexpr int OZ7_CHUNK_C = 256, OZ7_CHUNK_R = 512;
+constexpr int OZ5_CHUNK_C = 1488, OZ5_CHUNK_R = 2976;  // (exact to K' = 5461; 12 bytes times 2976 fit the workspace)
 
 // Products longer than one chunk: C = alpha sum_c op(A)(:, c) op(B)(c, :) + beta C, every
 // chunk FP64-accurate, the sum accumulated in FP64 through beta = 1.  digits: 5, 6, 7 or 10
@@ -736,7 +814,8 @@ cudaError_t launch_oz_chunked(int nprob, GemmDims dims, double alpha, GemmOperan
   // accurate (63 bits) and fewer, wider MMAs
   if (digits == NAO_OZ_DIGITS_FP64 && dims.K <= (REAL ? OZ7_CHUNK_R : OZ7_CHUNK_C)) digits = NAO_OZ_DIGITS_B128;
   const bool b128 = digits == NAO_OZ_DIGITS_B128;
-  const int chunk = b128 ? (REAL ? OZ7_CHUNK_R : OZ7_CHUNK_C) : (REAL ? OZ_CHUNK_R : OZ_CHUNK_C);
+  const int chunk = b128 ? (REAL ? OZ7_CHUNK_R : OZ7_CHUNK_C)
+                         : digits == NAO_OZ_DIGITS_FP64 ? (REAL ? OZ5_CHUNK_R : OZ5_CHUNK_C) : (REAL ? OZ_CHUNK_R : OZ_CHUNK_C);
   const size_t esz = REAL ? sizeof(double) : sizeof(z64);
   for (int k0 = 0; k0 < dims.K || k0 == 0; k0 += chunk) {
     GemmDims d = dims;
@@ -751,7 +830,7 @@ cudaError_t launch_oz_chunked(int nprob, GemmDims dims, double alpha, GemmOperan
       case 5: e = launch_oz<REAL, 5, 6>(nprob, d, alpha, a, b, bt, C, Cbs, Crs, Ccs, ws, err, st); break;
       case 6: e = launch_oz<REAL, 6, 6>(nprob, d, alpha, a, b, bt, C, Cbs, Crs, Ccs, ws, err, st); break;
       case 7: e = launch_oz<REAL, 7, 6>(nprob, d, alpha, a, b, bt, C, Cbs, Crs, Ccs, ws, err, st); break;
-      case OZ_S: e = launch_oz<REAL, OZ_S, 6>(nprob, d, alpha, a, b, bt, C, Cbs, Crs, Ccs, ws, err, st); break;
+      case NAO_OZ_DIGITS_FP64: e = launch_oz<REAL, 12, 5>(nprob, d, alpha, a, b, bt, C, Cbs, Crs, Ccs, ws, err, st); break;
       case NAO_OZ_DIGITS_B128: e = launch_oz<REAL, 9, 7>(nprob, d, alpha, a, b, bt, C, Cbs, Crs, Ccs, ws, err, st); break;
       default: return cudaErrorInvalidValue;
     }
@@ -768,7 +847,7 @@ bool zgemm_oz_supported(GemmDims dims) { return dims.M > 0 && dims.N > 0 && dims
 size_t zgemm_oz_workspace(int nprob, GemmDims dims) {
   const int Kc = dims.K < OZ_CHUNK_C ? dims.K : OZ_CHUNK_C;
   const int Mp = round_up(dims.M, OZ_BM), N2p = round_up(2 * dims.N, OZ_BN), K2p = round_up(2 * Kc, OZ_BK);
-  const size_t a = (size_t)nprob * OZ_S * Mp * K2p * 2, b = (size_t)nprob * OZ_S * N2p * K2p * 2;
+  const size_t a = (size_t)nprob * OZ_WS_PLANES * Mp * K2p * 2, b = (size_t)nprob * OZ_WS_PLANES * N2p * K2p * 2;
   return a + b + (size_t)nprob * (Mp + N2p) * sizeof(int) + 4096;
 }
 
@@ -783,7 +862,7 @@ bool dgemm_oz_supported(GemmDims dims) { return dims.M > 0 && dims.N > 0 && dims
 size_t dgemm_oz_workspace(int nprob, GemmDims dims) {
   const int Kc = dims.K < OZ_CHUNK_R ? dims.K : OZ_CHUNK_R;
   const int Mp = round_up(dims.M, OZ_BM), Np = round_up(dims.N, OZ_BN), Kp = round_up(Kc, OZ_BK);
-  return (size_t)nprob * OZ_S * ((size_t)Mp + Np) * Kp * 2 + (size_t)nprob * ((size_t)Mp + Np) * sizeof(int) + 4096;
+  return (size_t)nprob * OZ_WS_PLANES * ((size_t)Mp + Np) * Kp * 2 + (size_t)nprob * ((size_t)Mp + Np) * sizeof(int) + 4096;
 }
 
 cudaError_t launch_dgemm_oz(int nprob, GemmDims dims, double alpha, GemmOperand A, GemmOperand B, double beta, double* C,
