@@ -688,7 +688,7 @@ oz_gemm_kernel(int nprob, GemmDims dims, double alpha, double beta, const __nv_b
 #pragma unroll
         for (int a = 0; a < NEX; ++a) {
           const float gv = __uint_as_float(v[a][c]);
-          const long long ng = (long long)__float2int_rn(ldexpf(gv, DB * a - 30));
+          const long long ng = (long long)__float2int_rn(gv * __int_as_float((127 + DB * a - 30) << 23));  // gv 2^{DB a - 30}
           hi += ng * (1ll << (DB * (NEX - 1 - a)));
         }
         if (NEX < NACC) {
