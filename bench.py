@@ -169,14 +169,23 @@ class ClockSampler:
                 "reasons": sorted(reasons), "samples": len(sm)}
 
 
+def _overlaps_reduced(inp, m_mean):
+    """Overlap matrices that go through Eigen_HH(S): those with cut directions; where nothing is cut
+    X comes from the Cholesky factor (counted as no reduction, also for the ill-conditioned ones
+    that are reduced all the same)."""
+    return inp.nk if m_mean < inp.n else 0
+
+
 def _stage_flops(stage, inp, m_mean, nocc_mean):
     """Algorithmic FLOPs of one step for a traced stage (FP64, real-flop count)."""
-    n, ns, npb, nR, nk = inp.n, inp.nk, inp.nprob, inp.nR, inp.nk
+    n, ns, npb, nR, nk = inp.n, _overlaps_reduced(inp, m_mean), inp.nprob, inp.nR, inp.nk
     m = m_mean
     if stage == "hetrd":       # panel kernel: the Hermitian matvec half of 16/3 n^3 (digit products)
         return ns * 8.0 / 3.0 * n ** 3 + npb * 8.0 / 3.0 * m ** 3
     if stage == "hetrd_update":  # rank-2NB updates: the other half, tensor cores
         return ns * 8.0 / 3.0 * n ** 3 + npb * 8.0 / 3.0 * m ** 3
+    if stage == "overlap_chol":  # Cholesky factor and inverse, n^3 / 3 complex multiply-adds each
+        return nk * 16.0 / 3.0 * n ** 3
     if stage == "backtransform":  # Q Z with Q from n-1 complex reflectors: 8 n^2 per column
         return ns * 8.0 * n * n * m + npb * 8.0 * m ** 3
     if stage == "ortho_ns":    # Z (3I - Z^T Z)/2: two real n^3 GEMMs
@@ -206,15 +215,15 @@ def _panel_bytes(inp, m_mean):
     """Algorithmic DRAM bytes of the Householder reductions of one step: every column's
     Hermitian matrix-vector product reads the trailing matrix once in half storage (the
     lower triangle, FP64 complex: 16 B per entry, L^2 / 2 entries), i.e. 8 sum_L L^2 ~
-    (8/3) n^3 bytes per reduction (nk overlap matrices of order n, nprob H' of order m)."""
-    return 8.0 * (inp.nk * _sum_sq(inp.n) + inp.nprob * _sum_sq(m_mean))
+    (8/3) n^3 bytes per reduction (the reduced overlap matrices of order n, nprob H' of order m)."""
+    return 8.0 * (_overlaps_reduced(inp, m_mean) * _sum_sq(inp.n) + inp.nprob * _sum_sq(m_mean))
 
 
 def _digit_stream_bytes(inp, m_mean):
     """Bytes the digit form of the panel kernel streams by design: 8-bit digits of both
     triangles (8 digits x (re, im) = 16 B per entry, L^2 entries), 16 sum_L L^2 per matrix:
     twice the algorithmic bytes, the price of per-row digit scales."""
-    return 16.0 * (inp.nk * _sum_sq(inp.n) + inp.nprob * _sum_sq(m_mean))
+    return 16.0 * (_overlaps_reduced(inp, m_mean) * _sum_sq(inp.n) + inp.nprob * _sum_sq(m_mean))
 
 
 def _load_traffic(stage, units_per_launch):
@@ -802,8 +811,8 @@ def run_ours(args, rank, world, local_rank):
             hbm, hsrc = _hbm_peak()
             byts = _panel_bytes(inp, m_mean) * args.steps / max(dl, 1)
             achieved = byts / (per_launch_ms * 1e-3) / 1e9
-            roof = {"kernel": "hetrd_panel_kernel", "bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s",
-                    "frac": achieved / hbm, "traffic": _load_traffic(dname, (inp.nk + inp.nprob) / (dl / args.steps)),
+            roof = {"kernel": "hetrd_panel_mma_kernel", "bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s",
+                    "frac": achieved / hbm, "traffic": _load_traffic(dname, (_overlaps_reduced(inp, m_mean) + inp.nprob) / (dl / args.steps)),
                     "peak_source": hsrc, "algorithmic_bytes_per_launch": byts,
                     "algorithmic_bytes": "8 sum_L L^2 ~ (8/3) n^3 per reduction: the trailing matrix in half "
                                          "storage (FP64 complex) once per column",
