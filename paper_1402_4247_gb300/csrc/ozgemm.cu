@@ -32,7 +32,7 @@
 // n = 2000, H X 2.0 -> 1.4.  Contractions of 96 (256) terms with the twelve e4m3 planes instead of the nine
 // base-128 ones, which leave TMEM for two blocks per SM: rank-2k updates of n = 568, 128 problems 11.2
 // against 9.5 ms, density phase sums 7.0 against 5.2: hence the line at 256.
-// Pipeline: the digit tiles of each K step (16) arrive in one of three shared-memory stages
+// Pipeline: the digit tiles of each K step arrive in one of three shared-memory stages
 // by bulk asynchronous copies (TMA) issued by one producer thread; one thread issues the
 // MMAs and commits them to the stage's barrier.  Every wait is bounded (clock64; the
 // pipeline's waits by the context's nao_config.tc_wait_cycles); on timeout the block records
