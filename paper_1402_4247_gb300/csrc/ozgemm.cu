@@ -16,7 +16,7 @@
 //    and one TMEM accumulator per group keeps them;
 //  * three digit forms:
 //      e4m3, base 32, S = 12 (59 bits; e4m3 holds the integers up to 16): FP64 accuracy for more
-//        than 256 terms (512 real); all twelve groups exact to K' = 5461;
+//        than 176 terms (352 real); all twelve groups exact to K' = 5461;
 //      bf16, base 128, S = 9 (63 bits, exact to K' = 512): FP64 accuracy for shorter contractions;
 //      bf16, base 64, S = 5, 6, 7 (30 to 42 bits): terms that tolerate less.
 //    bf16 planes carry the digit's weight, A_s = d_s 2^{-b s}, B_t = d_t 2^{30 - b t}; the groups of
@@ -29,9 +29,10 @@
 // digits takes ~2070 cycles per 32 columns (16 MMAs, 60 KB); ten base-64 bf16 planes (55 products in
 // 31 MMAs, as accurate) took 2 x 2820 per 64 and wrote 1.7 times the bytes.  Measured (splits
 // included): 24 products of 301 x 257 x 420 625 -> 450 us; n = 568, 128 problems, H X 7.1 -> 5.5 ms;
-// n = 2000, H X 2.0 -> 1.4.  Contractions of 96 (256) terms with the twelve e4m3 planes instead of the nine
-// base-128 ones, which leave TMEM for two blocks per SM: rank-2k updates of n = 568, 128 problems 11.2
-// against 9.5 ms, density phase sums 7.0 against 5.2: hence the line at 256.
+// n = 2000, H X 2.0 -> 1.4.  Short contractions keep the nine base-128 planes, which leave TMEM for two
+// blocks per SM, one in its epilogue.  The line, us with nine base-128 / twelve e4m3 planes: 24 products of
+// 301 x 257 x K: K = 128 188 / 195, 160 231 / 222, 192 261 / 243, 256 322 / 289; 64 of 256 x 256 x K: 160 381 / 390,
+// 192 425 / 424, 256 520 / 496; one of 600 x 600 x K: 128 52 / 55, 160 60 / 60, 256 79 / 74.
 // Pipeline: the digit tiles of each K step arrive in one of three shared-memory stages
 // by bulk asynchronous copies (TMA) issued by one producer thread; one thread issues the
 // MMAs and commits them to the stage's barrier.  Every wait is bounded (clock64; the
@@ -812,6 +813,7 @@ cudaError_t launch_oz(int nprob, GemmDims dims, double alpha, GemmOperand A, Gem
 // K' <= OZ_MAX_K2 (real); base-128 digits K' <= 512.
 constexpr int OZ_CHUNK_C = OZ_MAX_K2 / 2, OZ_CHUNK_R = OZ_MAX_K2;
 constexpr int OZ7_CHUNK_C = 256, OZ7_CHUNK_R = 512;
+constexpr int OZ7_MAX_C = 176, OZ7_MAX_R = 352;  // longer FP64-accurate contractions take the e4m3 planes
 constexpr int OZ5_CHUNK_C = 1488, OZ5_CHUNK_R = 2976;  // (exact to K' = 5461; 12 bytes times 2976 fit the workspace)
 
 // Products longer than one chunk: C = alpha sum_c op(A)(:, c) op(B)(c, :) + beta C, every
@@ -821,9 +823,8 @@ template <bool REAL>
 cudaError_t launch_oz_chunked(int nprob, GemmDims dims, double alpha, GemmOperand A, GemmOperand B, double beta,
                               void* C, long long Cbs, long long Crs, long long Ccs, void* ws, int* err,
                               cudaStream_t st, int digits) {
-  // FP64-accurate contractions that fit one base-128 chunk take the nine base-128 planes: as
-  // accurate (63 bits) and fewer, wider MMAs
-  if (digits == NAO_OZ_DIGITS_FP64 && dims.K <= (REAL ? OZ7_CHUNK_R : OZ7_CHUNK_C)) digits = NAO_OZ_DIGITS_B128;
+  // short FP64-accurate contractions take the nine base-128 planes
+  if (digits == NAO_OZ_DIGITS_FP64 && dims.K <= (REAL ? OZ7_MAX_R : OZ7_MAX_C)) digits = NAO_OZ_DIGITS_B128;
   const bool b128 = digits == NAO_OZ_DIGITS_B128;
   const int chunk = b128 ? (REAL ? OZ7_CHUNK_R : OZ7_CHUNK_C)
                          : digits == NAO_OZ_DIGITS_FP64 ? (REAL ? OZ5_CHUNK_R : OZ5_CHUNK_C) : (REAL ? OZ_CHUNK_R : OZ_CHUNK_C);
