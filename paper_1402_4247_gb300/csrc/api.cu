@@ -189,6 +189,7 @@ struct GenEigPlan {
   size_t oNs2, oNc2;
   // Cholesky route of the overlap: failures, norms, orders left for Eigen_HH
   size_t oCf, oCp, oCs;
+  bool md_own;  // the panel digits have an array of their own
   size_t bytes;
 };
 
@@ -241,7 +242,10 @@ GenEigPlan plan_gen_eig(int n, int nprob, int nSe, bool use_tc, int B2, bool spl
   // 8-bit digit planes of the Householder trailing matrix (tensor-core product method)
   W.oDig = P.take<char>(use_tc ? hetrd_digits_bytes(n, nmax, NAO_HT_DIGITS_FP64) : 16);
   W.oErow = P.take<int>((size_t)(n > 1 ? n - 1 : 1) * nmax);
-  W.oMd = P.take<char>(use_tc ? hetrd_panel_bytes(n, nmax) : 16);  // and of its panels
+  // and of its panels: in the back-transformation's arrays (oVf .. oW2), which hold nothing while a
+  // matrix is reduced; with Parts 3-4 in halves in the half's slice of oVf, where that is enough
+  W.md_own = split && use_tc && hetrd_panel_bytes(n, 1) > (size_t)n * ncolv * sizeof(z64);
+  W.oMd = W.md_own ? P.take<char>(hetrd_panel_bytes(n, nmax)) : W.oVf;
   const size_t b2 = B2 > 0 ? (size_t)B2 : 0;
   const size_t sq = B2 > 0 ? (size_t)sbr_q2_count(n, B2) : 0;
   W.oSVT = P.take<z64>(b2 * n * nmax + 1);
@@ -1055,7 +1059,7 @@ int nao_gen_eig_sized(nao_ctx* ctx, int n, int nprob, const nao_c128* H, const n
       h.stH = stH + p0;
       h.ozws = oz_h;
       h.digp = dig_h;
-      h.mdp = p0 ? (char*)mdp + hetrd_panel_bytes(n, p0) : (char*)mdp;
+      h.mdp = !W.md_own ? (char*)h.Vf : p0 ? (char*)mdp + hetrd_panel_bytes(n, p0) : (char*)mdp;
       h.erowp = erowp + (size_t)p0 * (n > 1 ? n - 1 : 1);
       h.ns2 = ns2f + p0;
       h.nc2 = nc2 + p0;

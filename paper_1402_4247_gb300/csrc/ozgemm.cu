@@ -47,7 +47,7 @@
 
 namespace {
 
-constexpr int OZ_WS_PLANES = 10;     // bf16 planes that the workspace holds (12 e4m3 planes take less)
+constexpr int OZ_WS_PLANES = 9;      // bf16 planes that the workspace holds (12 e4m3 planes take less)
 constexpr int OZ_BM = 128;           // tile rows (C'' rows)
 constexpr int OZ_BN = 64;            // tile columns (C'' columns = 32 complex columns); B plane tile rows
 constexpr int OZ_BK = 16;            // K' per MMA step (bf16 digits; 32 with e4m3 digits: the same bytes)
@@ -689,7 +689,7 @@ oz_gemm_kernel(int nprob, GemmDims dims, double alpha, double beta, const __nv_b
       for (int c = 0; c < CW; ++c) {
         if (DB == 5) {
           // group a counts in units of 2^{-8 - 5 a} and is exact (2^8 a product, 12 in a group, K' <=
-          // 2976: below 2^24): two words of six groups each, in units of 2^-33 and 2^-63
+          // 2688: below 2^24): two words of six groups each, in units of 2^-33 and 2^-63
           // (|.| < 2^50), joined with the low word rounded at least 2^-60 below the result
           long long hi = 0, lo = 0;
 #pragma unroll
@@ -814,7 +814,7 @@ cudaError_t launch_oz(int nprob, GemmDims dims, double alpha, GemmOperand A, Gem
 constexpr int OZ_CHUNK_C = OZ_MAX_K2 / 2, OZ_CHUNK_R = OZ_MAX_K2;
 constexpr int OZ7_CHUNK_C = 256, OZ7_CHUNK_R = 512;
 constexpr int OZ7_MAX_C = 176, OZ7_MAX_R = 352;  // longer FP64-accurate contractions take the e4m3 planes
-constexpr int OZ5_CHUNK_C = 1488, OZ5_CHUNK_R = 2976;  // (exact to K' = 5461; 12 bytes times 2976 fit the workspace)
+constexpr int OZ5_CHUNK_C = 1344, OZ5_CHUNK_R = 2688;  // (exact to K' = 5461; 12 bytes x 2688 = 18 x OZ_MAX_K2)
 
 // Products longer than one chunk: C = alpha sum_c op(A)(:, c) op(B)(c, :) + beta C, every
 // chunk FP64-accurate, the sum accumulated in FP64 through beta = 1.  digits: 5, 6, 7 or 10

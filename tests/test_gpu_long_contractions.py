@@ -1,7 +1,7 @@
 """Tensor-core products of more than 176 terms (352 real), formed from e4m3 digits (GPU only): operands
 of 20-bit integers, whose digits beyond the fifth are zero and whose products and sums are exact
 in FP64, must come back exactly.  Orders around the tiles (128 rows, 16 columns), the K steps of 32
-with both halves of a complex contraction, the chunks of 1488, and the largest digit sums."""
+with both halves of a complex contraction, the chunks of 1344, and the largest digit sums."""
 import numpy as np
 import pytest
 
@@ -23,7 +23,7 @@ def ctx():
 @pytest.mark.parametrize("largest", [False, True], ids=["random", "largest"])
 @pytest.mark.parametrize("P,M,N,K,tA,tB", [
     (1, 33, 18, 176, 0, 0), (2, 131, 17, 177, 2, 1), (1, 1, 1, 257, 0, 0), (2, 127, 15, 264, 0, 1), (3, 128, 16, 272, 2, 0), (1, 129, 17, 273, 1, 2), (2, 31, 33, 288, 0, 2),
-    (1, 300, 100, 289, 2, 2), (1, 16, 257, 1487, 0, 0), (1, 130, 40, 1488, 2, 1), (1, 65, 31, 1489, 1, 0), (1, 20, 18, 2990, 0, 2)])
+    (1, 300, 100, 289, 2, 2), (1, 16, 257, 1343, 0, 0), (1, 130, 40, 1344, 2, 1), (1, 65, 31, 1345, 1, 0), (1, 20, 18, 2700, 0, 2)])
 def test_integer_products(ctx, P, M, N, K, tA, tB, largest):
     from paper_1402_4247_gb300.nao import NAO_GEMM_TC
     rng = np.random.Generator(np.random.PCG64(M + 10 * N + 100 * K))
