@@ -393,7 +393,15 @@ stebz_kernel(int n, const int32_t* __restrict__ size, const double* __restrict__
   wslot[(size_t)p * n + j] = lam;
 }
 
-// Kernel 1b: FP64 bisection of the queued eigenvalues of all problems, one thread per queue
+// Lanes per queued eigenvalue: BQ_LANES, or as many more (a power of two, 32 at most) as leave a
+// short queue's warps a scheduler each (warps of them), and never more than the launch has threads for
+__host__ __device__ inline int bisect_lanes(long long cnt, long long threads, long long warps) {
+  int ln = BQ_LANES;
+  while (ln < 32 && cnt * ln <= warps * 16 && 2 * cnt * ln <= threads) ln *= 2;
+  return ln;
+}
+
+// Kernel 1b: FP64 bisection of the queued eigenvalues of all problems, bisect_lanes lanes per queue
 // entry, so that the warps are full however few entries each problem has.  An entry carries
 // its problem, slot, split block and verified bracket; d and the split e^2 are read from
 // global memory (each lane streams its own problem's arrays).  (Switching a lane to Newton
@@ -402,14 +410,12 @@ stebz_kernel(int n, const int32_t* __restrict__ size, const double* __restrict__
 __global__ void __launch_bounds__(SZ_THREADS)
 stebz_bisect_kernel(int n, const double* __restrict__ dbase, long long strideV, const double* __restrict__ e2g,
                     const double* __restrict__ tng, double* __restrict__ wslot, const int* __restrict__ qcount,
-                    const int4* __restrict__ qent, const double* __restrict__ qlo, const double* __restrict__ qhi) {
+                    const int4* __restrict__ qent, const double* __restrict__ qlo, const double* __restrict__ qhi, int warps) {
   // LN lanes per entry: each step counts at LN interior points of the bracket, one per lane,
   // and keeps the sub-interval that holds the eigenvalue (log2(LN + 1) bits per step instead of
-  // one): the dependent chain of steps sets this kernel's time.  BQ_LANES, or as many more (32 at
-  // most) as leave a short queue's warps a scheduler each (608 on this GPU)
+  // one): the dependent chain of steps sets this kernel's time
   const int cnt = *qcount;
-  int LN = BQ_LANES;
-  while (LN < 32 && cnt * LN <= 608 * 16) LN *= 2;
+  const int LN = bisect_lanes(cnt, gridDim.x * blockDim.x, warps);
   const int gt = blockIdx.x * blockDim.x + threadIdx.x;
   const int q = gt / LN, sub = gt % LN;
   if (q >= cnt) return;  // uniform over the entry's lanes
@@ -1266,14 +1272,20 @@ size_t stein_scratch_doubles(int n, int nprob) {
          ((size_t)n * nprob + 1) / 2 + 1 + nprob + 2;
 }
 
-// lanes per eigenvalue of stebz_multi_kernel: as many as leave each warp a scheduler of its own (4
-// per SM), 16 at most; 1: kernels 1 and 1b
-static int stebz_lanes(int n, int nprob) {
+// SMs of the current device, 0 when the query fails
+static int sm_count() {
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
     cudaGetLastError();
-    return 1;
+    return 0;
   }
+  return sms;
+}
+
+// lanes per eigenvalue of stebz_multi_kernel: as many as leave each warp a scheduler of its own (4
+// per SM), 16 at most; 1: kernels 1 and 1b
+static int stebz_lanes(int n, int nprob) {
+  const int sms = sm_count();
   int ln = 16;
   while (ln > 2 && (size_t)n * nprob * ln > (size_t)sms * 4 * 32) ln /= 2;
   return ln > 2 ? ln : 1;  // (two lanes were slower: n = 211, 24 problems 1.75 ms against 1.37)
@@ -1317,7 +1329,7 @@ cudaError_t launch_stein(int n, int nprob, const int32_t* size, const double* d,
     if (err != cudaSuccess) return err;
     stebz_bisect_kernel<<<(unsigned)((cap * BQ_LANES + SZ_THREADS - 1) / SZ_THREADS), SZ_THREADS, 0, st>>>(n, d, strideV, e2g, tng,
                                                                                                wslot, qcount, qent, qlo,
-                                                                                               qhi);
+                                                                                               qhi, 4 * sm_count());
     err = cudaGetLastError();
     if (err != cudaSuccess) return err;
   }
