@@ -176,8 +176,9 @@ int nao_bloch_sum(nao_ctx* ctx, int n, int nR, const int32_t* R, int nmat, const
  * X = U_m diag(s_m^{-1/2}) over the m eigenvalues s_j >= s_cut; H' = X^H H X;
  * Eigen_HH(H') -> eps, V; C = X V.  Where every direction of S is kept and S is well
  * conditioned ((tr S / n) tr(S^{-1}) <= 1e6, decided on the device per matrix; NAO_GEMM_TC, FP64 or
- * mixed with refinement 0, default settings of Eigen_HH), X = L^{-H} from S = L L^H takes the
- * place of Eigen_HH(S): the same eps, and C up to the free phase of each column.
+ * mixed with refinement 0, default settings of Eigen_HH), X = L^{-H} from S = L L^H (FP64-accurate
+ * products in every mode) takes the place of Eigen_HH(S): the same eps, and C up to the free
+ * phase of each column.
  *   n         basis size (>= 1); nprob problems (>= 1)
  *   H         complex128 [nprob][n][n] Hermitian (lower triangle read)
  *   S         complex128 [nS][n][n] Hermitian positive semi-definite (lower triangle read)

@@ -568,10 +568,13 @@ double* ns_second(nao_ctx* ctx, int n, int nprob, const int32_t* size, const int
 }
 
 // Part 2 without Eigen_HH (csrc/chol.cu): X = L^{-H} of every overlap matrix, S given full in X;
-// size_eff says which of them still need Eigen_HH(S).  Y, fail, part: scratch.  digits: planes of the
-// products (the mixed mode's X is as accurate as its back-transformations).
+// size_eff says which of them still need Eigen_HH(S).  Y, fail, part: scratch.  FP64-accurate products
+// in the mixed mode too: a backward error u |S| of the factor leaves X^H S X - 1 ~ u cond(S), where the
+// eigenvector route, whose reduction of S is FP64-accurate in every mode, has u sqrt(cond(S)) from
+// its back-transformation.  (n = 300, (tr S / n) tr S^-1 = 9.4e5, 36-bit products here: C^H S C - 1
+// 1.0e-7 against 3.4e-8; 30 bits: 8.6e-6 against 2.1e-6.)
 cudaError_t overlap_cholesky(nao_ctx* ctx, int n, int nS, const int32_t* size, const z64* S, z64* X, double s_cut, z64* Y,
-                             int* fail, double* part, int32_t* size_eff, void* ozws, cudaStream_t st, int digits) {
+                             int* fail, double* part, int32_t* size_eff, void* ozws, cudaStream_t st) {
   const long long snn = (long long)n * n;
   // 32 columns per step while a step is bound by its launches and its diagonal block (29 us of FP64
   // at 32 columns, 155 us at 64), 64 once the passes over the trailing matrices (~27 ns per
@@ -594,12 +597,12 @@ cudaError_t overlap_cholesky(nao_ctx* ctx, int n, int nS, const int32_t* size, c
     }
     e = run_zgemm(ctx, "overlap_chol", nS, GemmDims{n, w, w, nullptr, nullptr, nullptr, 0}, 1.0,
                   GemmOperand{P, snn, 1, n, 0, nullptr}, GemmOperand{Y, (long long)B * B, 1, B, 1, nullptr}, 0.0, P, snn, 1,
-                  n, ozws, st, digits);  // times Y^H, in place (the operands are split first)
+                  n, ozws, st);  // times Y^H, in place (the operands are split first)
     if (e != cudaSuccess) return e;
     if (rest == 0) break;
     e = run_zgemm(ctx, "overlap_chol", nS, GemmDims{n, rest, w, nullptr, nullptr, nullptr, 0}, -1.0,
                   GemmOperand{P, snn, 1, n, 0, nullptr}, GemmOperand{P + j0 + w, snn, n, 1, 1, nullptr}, 1.0,
-                  X + (size_t)(j0 + w) * n, snn, 1, n, ozws, st, digits);
+                  X + (size_t)(j0 + w) * n, snn, 1, n, ozws, st);
     if (e != cudaSuccess) return e;
   }
   NaoStage stage_(ctx, "overlap_chol", st, 2);
@@ -929,7 +932,7 @@ int nao_gen_eig_sized(nao_ctx* ctx, int n, int nprob, const nao_c128* H, const n
   if (chol) {
     int32_t* se = (int32_t*)(ws + W.oCs);
     NAO_CUDA_TRY(ctx, overlap_cholesky(ctx, n, nSe, s_size, (const z64*)S, X, s_cut, Tw, (int*)(ws + W.oCf),
-                                       (double*)(ws + W.oCp), se, ozws, st, dig));
+                                       (double*)(ws + W.oCp), se, ozws, st));
     sz = on = se;
   }
   if (B2 > 0)
