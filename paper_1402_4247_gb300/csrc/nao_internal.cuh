@@ -309,8 +309,8 @@ cudaError_t launch_ns_correct(int n, int nprob, const int32_t* size, const int32
 // + beta C with real alpha, beta.  Long contractions run as chunks whose FP32 group sums stay
 // exact, accumulated in FP64.  ws: zgemm_oz_workspace bytes; err: the context's dev_flags
 // (err[NAO_FLAG_TIMEOUT] set to 1 if a bounded wait expired; the bound is the long long at err +
-// NAO_FLAG_WAIT).  digits: NAO_OZ_DIGITS_FP64 (FP64 accuracy: nine base-128 bf16 planes, 63 bits, up to
-// 176 terms, 352 real, else twelve base-32 e4m3 planes, 59 bits, in chunks of 1344, 2688 real), or 5, 6, 7
+// NAO_FLAG_WAIT).  digits: NAO_OZ_DIGITS_FP64 (63-bit operands: nine base-128 bf16 planes up to
+// 256 terms, 512 real, else thirteen base-32 e4m3 planes in chunks of 1232, 2464 real), or 5, 6, 7
 // base-64 planes (30, 36, 42 bits: 15, 21, 28 products) for terms that tolerate less;
 // NAO_OZ_DIGITS_B128: the nine base-128 planes in any case (chunks of 256, 512 real).
 constexpr int NAO_OZ_DIGITS_FP64 = 10;

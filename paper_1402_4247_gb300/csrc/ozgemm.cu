@@ -15,8 +15,8 @@
 //    group s + t share a power of two, so a group's FP32 sums are exact integers while below 2^24,
 //    and one TMEM accumulator per group keeps them;
 //  * three digit forms:
-//      e4m3, base 32, S = 12 (59 bits; e4m3 holds the integers up to 16): FP64 accuracy for more
-//        than 176 terms (352 real); all twelve groups exact to K' = 5461;
+//      e4m3, base 32, S = 13 (63 bits; e4m3 holds the integers up to 16): FP64 accuracy for more
+//        than 256 terms (512 real); all thirteen groups exact to K' = 5041;
 //      bf16, base 128, S = 9 (63 bits, exact to K' = 512): FP64 accuracy for shorter contractions;
 //      bf16, base 64, S = 5, 6, 7 (30 to 42 bits): terms that tolerate less.
 //    bf16 planes carry the digit's weight, A_s = d_s 2^{-b s}, B_t = d_t 2^{30 - b t}; the groups of
@@ -25,14 +25,18 @@
 //    by the rows' and columns' powers of two; real alpha, beta.
 // What bounds it: an MMA with A from shared memory costs max(N / 2, ~48) cycles for K = 16 bf16 or 32
 // e4m3 columns (measured, N = 32 .. 256), so the digit planes t of B are stacked into operands of up
-// to 256 rows; the operands' shared-memory traffic then sets the pace.  A K step of 32 with e4m3
-// digits takes ~2070 cycles per 32 columns (16 MMAs, 60 KB); ten base-64 bf16 planes (55 products in
-// 31 MMAs, as accurate) took 2 x 2820 per 64 and wrote 1.7 times the bytes.  Measured (splits
-// included): 24 products of 301 x 257 x 420 625 -> 450 us; n = 568, 128 problems, H X 7.1 -> 5.5 ms;
-// n = 2000, H X 2.0 -> 1.4.  Short contractions keep the nine base-128 planes, which leave TMEM for two
-// blocks per SM, one in its epilogue.  The line, us with nine base-128 / twelve e4m3 planes: 24 products of
-// 301 x 257 x K: K = 128 188 / 195, 160 231 / 222, 192 261 / 243, 256 322 / 289; 64 of 256 x 256 x K: 160 381 / 390,
-// 192 425 / 424, 256 520 / 496; one of 600 x 600 x K: 128 52 / 55, 160 60 / 60, 256 79 / 74.
+// to 256 rows; the operands' shared-memory traffic then sets the pace.  Thirteen e4m3 planes: 91
+// products in 18 MMAs and 65 KB per K step of 32 and 32 columns, against 55 products in 31 MMAs per 16 and
+// 64 of ten base-64 bf16 planes (60 bits), which also wrote 1.5 times the bytes.  Measured (splits
+// included), ten bf16 -> thirteen e4m3: 24 products of 301 x 257 x 420 625 -> 497 us; n = 568, 128 problems,
+// H X 7.1 -> 6.0 ms; n = 2000, H X 2.0 -> 1.5.  (Twelve planes, 59 bits: 450 us, 5.5 and 1.4 ms, but their dropped
+// products doubled the residuals of eigenvectors: n = 400, S = 1, median |H c - c e| 3.9 eps |H| with the
+// ten, 5.3 with twelve, 2.0 with thirteen; products of graded operands at K = 200 were 35 times less
+// accurate than nine base-128 planes.)
+// The line (one base-128 chunk, 256 terms): nine base-128 planes drop products from 2^-77 on, thirteen
+// e4m3 from 2^-71, and leave TMEM for two blocks per SM, one in its epilogue.  us with nine / thirteen planes at
+// K = 64, 128, 256: 24 products of 301 x 257 128 / 151, 187 / 213, 323 / 318; 64 of 256 x 256 213 / 297, 310 / 379, 520 / 543;
+// one of 600 x 600 37 / 44, 52 / 57, 79 / 78.
 // Pipeline: the digit tiles of each K step arrive in one of three shared-memory stages
 // by bulk asynchronous copies (TMA) issued by one producer thread; one thread issues the
 // MMAs and commits them to the stage's barrier.  Every wait is bounded (clock64; the
@@ -47,7 +51,7 @@
 
 namespace {
 
-constexpr int OZ_WS_PLANES = 9;      // bf16 planes that the workspace holds (12 e4m3 planes take less)
+constexpr int OZ_WS_PLANES = 9;      // bf16 planes that the workspace holds (13 e4m3 planes take less)
 constexpr int OZ_BM = 128;           // tile rows (C'' rows)
 constexpr int OZ_BN = 64;            // tile columns (C'' columns = 32 complex columns); B plane tile rows
 constexpr int OZ_BK = 16;            // K' per MMA step (bf16 digits; 32 with e4m3 digits: the same bytes)
@@ -62,7 +66,7 @@ constexpr int OZ_SHORT_KSTEPS = 16;
 constexpr int OZ_THREADS = 256;
 __host__ __device__ constexpr int oz_threads(int DB) { return DB == 5 ? 2 * OZ_THREADS : OZ_THREADS; }
 constexpr long long OZ_WAIT_CYCLES = NAO_TC_WAIT_DEFAULT;  // ~2 s at 2 GHz
-constexpr int OZ_MAX_K2 = 1792;      // 2K bound for exact FP32 group sums (group 8: 9 2^10 per k)
+constexpr int OZ_MAX_K2 = 1792;      // 2K bound for exact FP32 sums of base-64 digits (the seventh group: 9 2^10 per term)
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -177,31 +181,38 @@ __device__ __forceinline__ uint32_t oz_bf16_bits(int d, int k) {
 }
 
 // the digits of the entries q(0), q(1), .. of a lane's 16-byte chunk: plane s's chunk in pk[s].
-// bf16 (DB 6 or 7): 8 entries d 2^{scale0 - DB s}.  e4m3 (DB = 5, S = 12): 16 entries d; the balanced digits
-// d + 16 are the 5-bit fields of q + 16 sum_s 32^s (the top one up to 32), taken for two entries
-// at a time from words that hold three fields of each in their halves, as f16 1024 + u - 1040
+// bf16 (DB 6 or 7): 8 entries d 2^{scale0 - DB s}.  e4m3 (DB = 5, S = 13, |q| < 2^63): 16 entries d; the
+// balanced digits d + 16 of q mod 2^60 are the 5-bit fields of (q mod 2^60) + 16 sum_s 32^s, the carry
+// goes to the top digit q >> 60 (|.| <= 8); taken for two entries at a time from words that hold
+// three fields of each in their halves, as f16 1024 + u - 1040
 template <int S, int DB, class Q>
 __device__ __forceinline__ void oz_pack(uint32_t (&pk)[S][4], int scale0, Q q) {
   if constexpr (DB == 5) {
-    static_assert(S == 12, "four words of three 5-bit digits");
+    static_assert(S == 13, "the top digit and four words of three 5-bit digits");
+    constexpr unsigned long long low = (1ull << 60) - 1, bias = 0x842108421084210ull;  // 16 in each of the twelve fields
+    auto half2 = [](uint32_t u) {  // two fields d + 16 as e4m3
+      u |= 0x64006400u;            // 1024 + (d + 16) in f16
+      const __half2 x = __hsub2(*(const __half2*)&u, __half2{__ushort_as_half(0x6410), __ushort_as_half(0x6410)});
+      return (uint32_t)__nv_cvt_halfraw2_to_fp8x2(*(const __half2_raw*)&x, __NV_SATFINITE, __NV_E4M3);
+    };
 #pragma unroll
     for (int w = 0; w < 4; ++w)
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        const unsigned long long bias = 0x842108421084210ull;  // 16 in each of the twelve 5-bit fields
-        const unsigned long long z0 = (unsigned long long)q(4 * w + 2 * h) + bias, z1 = (unsigned long long)q(4 * w + 2 * h + 1) + bias;
+        const long long q0 = q(4 * w + 2 * h), q1 = q(4 * w + 2 * h + 1);
+        const unsigned long long z0 = ((unsigned long long)q0 & low) + bias, z1 = ((unsigned long long)q1 & low) + bias;
+        const uint32_t t0 = (uint32_t)((q0 >> 60) + (long long)(z0 >> 60) + 16), t1 = (uint32_t)((q1 >> 60) + (long long)(z1 >> 60) + 16);
+        const uint32_t top = half2(t0 | t1 << 16);
+        pk[0][w] = h ? pk[0][w] | top << 16 : top;
 #pragma unroll
-        for (int part = 0; part < 4; ++part) {  // digits 3 part .. 3 part + 2
+        for (int part = 0; part < 4; ++part) {  // digits 3 part + 1 .. 3 part + 3
           const int sh = 45 - 15 * part;
-          const uint32_t keep = part ? 0x7fffu : 0xffffu;
-          const uint32_t y = ((uint32_t)(z0 >> sh) & keep) | ((uint32_t)(z1 >> sh) & keep) << 16;
+          const uint32_t y = ((uint32_t)(z0 >> sh) & 0x7fffu) | ((uint32_t)(z1 >> sh) & 0x7fffu) << 16;
 #pragma unroll
           for (int k = 0; k < 3; ++k) {
-            const uint32_t field = part == 0 && k == 0 ? 0x003f003fu : 0x001f001fu;
-            const uint32_t u = ((y >> (10 - 5 * k)) & field) | 0x64006400u;  // 1024 + (d + 16) in f16
-            const __half2 x = __hsub2(*(const __half2*)&u, __half2{__ushort_as_half(0x6410), __ushort_as_half(0x6410)});
-            const uint32_t b = __nv_cvt_halfraw2_to_fp8x2(*(const __half2_raw*)&x, __NV_SATFINITE, __NV_E4M3);
-            pk[3 * part + k][w] = h ? pk[3 * part + k][w] | b << 16 : b;
+            const uint32_t b = half2((y >> (10 - 5 * k)) & 0x001f001fu);
+            uint32_t& o = pk[1 + 3 * part + k][w];
+            o = h ? o | b << 16 : b;
           }
         }
       }
@@ -364,7 +375,7 @@ __global__ void __launch_bounds__(256) oz_split(int nprob, GemmDims dims, GemmOp
           const z64 z = ((const z64*)xb)[at(k)];
           v = h ? z.y : z.x;
         }
-        const long long q = oz_fixed<S, DB>(v, DB == 5 ? ex + 1 : ex);
+        const long long q = oz_fixed<S, DB>(v, DB == 5 ? ex + 2 : ex);
         return neg ? -q : q;
       });
       const int g2 = ng + g;
@@ -400,7 +411,7 @@ __global__ void __launch_bounds__(256) oz_split(int nprob, GemmDims dims, GemmOp
           neg = hi && X.conj != 0;  // conj: Im z enters with the opposite sign
         }
       }
-      const long long q = oz_fixed<S, DB>(v, DB == 5 ? ex + 1 : ex);
+      const long long q = oz_fixed<S, DB>(v, DB == 5 ? ex + 2 : ex);
       return neg ? -q : q;
     });
 #pragma unroll
@@ -486,7 +497,7 @@ oz_gemm_kernel(int nprob, GemmDims dims, double alpha, double beta, const __nv_b
   constexpr int STAGE = S * (OZ_TILE_A + TILE_B);     // bytes per pipeline stage
   constexpr int kUnitExp = DB * (NEX - 1) - 30;       // an accumulator's value in units of the last exact
                                                       // group: v 2^kUnitExp
-  constexpr int kExp = DB == 5 ? -33 : -DB * (NEX + 1);  // the output is t 2^{e_i + f_j + kExp - sh}
+  constexpr int kExp = DB == 5 ? -31 : -DB * (NEX + 1);  // the output is t 2^{e_i + f_j + kExp - sh}
   extern __shared__ __align__(1024) unsigned char oz_smem[];
   __shared__ uint64_t full_bar[NST], empty_bar[NST], done_bar;
   __shared__ uint32_t tbase;
@@ -688,18 +699,20 @@ oz_gemm_kernel(int nprob, GemmDims dims, double alpha, double beta, const __nv_b
 #pragma unroll
       for (int c = 0; c < CW; ++c) {
         if (DB == 5) {
-          // group a counts in units of 2^{-8 - 5 a} and is exact (2^8 a product, 12 in a group, K' <=
-          // 2688: below 2^24): two words of six groups each, in units of 2^-33 and 2^-63
-          // (|.| < 2^50), joined with the low word rounded at least 2^-60 below the result
+          // group a counts in units of 2^{-6 - 5 a} and is exact (2^8 a product, 13 in a group, K' <=
+          // 2464: below 2^24): two words of six and seven groups, in units of 2^-31 and 2^-66
+          // (|.| < 2^50 and 2^55), joined with the low word rounded at least 2^-60 below the result
+          constexpr int NHI = 6, NLO = NACC - NHI, D = DB * NLO;  // (D: bits between the two units)
           long long hi = 0, lo = 0;
 #pragma unroll
-          for (int a = 0; a < NACC / 2; ++a) {
-            hi += (long long)__float2int_rn(__uint_as_float(v[a][c])) * (1ll << (5 * (NACC / 2 - 1 - a)));
-            lo += (long long)__float2int_rn(__uint_as_float(v[NACC / 2 + a][c])) * (1ll << (5 * (NACC / 2 - 1 - a)));
-          }
+          for (int a = 0; a < NHI; ++a)
+            hi += (long long)__float2int_rn(__uint_as_float(v[a][c])) * (1ll << (5 * (NHI - 1 - a)));
+#pragma unroll
+          for (int a = 0; a < NLO; ++a)
+            lo += (long long)__float2int_rn(__uint_as_float(v[NACC - NLO + a][c])) * (1ll << (5 * (NLO - 1 - a)));
           const unsigned long long ah = hi < 0 ? 0ull - (unsigned long long)hi : (unsigned long long)hi;
-          const int s = min(max(__clzll((long long)ah) - 3, 0), 30);
-          t[c] = (long long)((unsigned long long)hi << s) + (s == 30 ? lo : (lo + (1ll << (29 - s))) >> (30 - s));
+          const int s = min(max(__clzll((long long)ah) - 3, 0), D);
+          t[c] = (long long)((unsigned long long)hi << s) + (s == D ? lo : (lo + (1ll << (D - 1 - s))) >> (D - s));
           sh[c] = s;
           continue;
         }
@@ -813,18 +826,18 @@ cudaError_t launch_oz(int nprob, GemmDims dims, double alpha, GemmOperand A, Gem
 // K' <= OZ_MAX_K2 (real); base-128 digits K' <= 512.
 constexpr int OZ_CHUNK_C = OZ_MAX_K2 / 2, OZ_CHUNK_R = OZ_MAX_K2;
 constexpr int OZ7_CHUNK_C = 256, OZ7_CHUNK_R = 512;
-constexpr int OZ7_MAX_C = 176, OZ7_MAX_R = 352;  // longer FP64-accurate contractions take the e4m3 planes
-constexpr int OZ5_CHUNK_C = 1344, OZ5_CHUNK_R = 2688;  // (exact to K' = 5461; 12 bytes x 2688 = 18 x OZ_MAX_K2)
+constexpr int OZ5_CHUNK_C = 1232, OZ5_CHUNK_R = 2464;  // (exact to K' = 5041; 13 bytes x 2464 <= 18 x OZ_MAX_K2)
+static_assert((OZ5_CHUNK_R + 31) / 32 * 32 * 13 <= 2 * OZ_WS_PLANES * OZ_MAX_K2, "the workspace of bf16 planes holds them");
 
 // Products longer than one chunk: C = alpha sum_c op(A)(:, c) op(B)(c, :) + beta C, every
-// chunk FP64-accurate, the sum accumulated in FP64 through beta = 1.  digits: 5, 6, 7 or 10
-// base-64 planes, or NAO_OZ_DIGITS_B128 (nine base-128 planes, 63 bits).
+// chunk FP64-accurate, the sum accumulated in FP64 through beta = 1.  digits: 5, 6 or 7
+// base-64 planes, NAO_OZ_DIGITS_FP64, or NAO_OZ_DIGITS_B128 (nine base-128 planes, 63 bits).
 template <bool REAL>
 cudaError_t launch_oz_chunked(int nprob, GemmDims dims, double alpha, GemmOperand A, GemmOperand B, double beta,
                               void* C, long long Cbs, long long Crs, long long Ccs, void* ws, int* err,
                               cudaStream_t st, int digits) {
-  // short FP64-accurate contractions take the nine base-128 planes
-  if (digits == NAO_OZ_DIGITS_FP64 && dims.K <= (REAL ? OZ7_MAX_R : OZ7_MAX_C)) digits = NAO_OZ_DIGITS_B128;
+  // FP64-accurate contractions that fit one base-128 chunk take the nine base-128 planes
+  if (digits == NAO_OZ_DIGITS_FP64 && dims.K <= (REAL ? OZ7_CHUNK_R : OZ7_CHUNK_C)) digits = NAO_OZ_DIGITS_B128;
   const bool b128 = digits == NAO_OZ_DIGITS_B128;
   const int chunk = b128 ? (REAL ? OZ7_CHUNK_R : OZ7_CHUNK_C)
                          : digits == NAO_OZ_DIGITS_FP64 ? (REAL ? OZ5_CHUNK_R : OZ5_CHUNK_C) : (REAL ? OZ_CHUNK_R : OZ_CHUNK_C);
@@ -842,7 +855,7 @@ cudaError_t launch_oz_chunked(int nprob, GemmDims dims, double alpha, GemmOperan
       case 5: e = launch_oz<REAL, 5, 6>(nprob, d, alpha, a, b, bt, C, Cbs, Crs, Ccs, ws, err, st); break;
       case 6: e = launch_oz<REAL, 6, 6>(nprob, d, alpha, a, b, bt, C, Cbs, Crs, Ccs, ws, err, st); break;
       case 7: e = launch_oz<REAL, 7, 6>(nprob, d, alpha, a, b, bt, C, Cbs, Crs, Ccs, ws, err, st); break;
-      case NAO_OZ_DIGITS_FP64: e = launch_oz<REAL, 12, 5>(nprob, d, alpha, a, b, bt, C, Cbs, Crs, Ccs, ws, err, st); break;
+      case NAO_OZ_DIGITS_FP64: e = launch_oz<REAL, 13, 5>(nprob, d, alpha, a, b, bt, C, Cbs, Crs, Ccs, ws, err, st); break;
       case NAO_OZ_DIGITS_B128: e = launch_oz<REAL, 9, 7>(nprob, d, alpha, a, b, bt, C, Cbs, Crs, Ccs, ws, err, st); break;
       default: return cudaErrorInvalidValue;
     }
