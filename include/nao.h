@@ -48,12 +48,14 @@ enum { NAO_FP64 = 0, NAO_MIXED_TF32 = 1, NAO_MIXED_BF16X3 = 2 };
 /* How the FP64 matrix products of the band step are computed (both FP64-accurate). */
 enum {
   NAO_GEMM_FP64 = 0,  /* FP64 FMA on the CUDA cores                                        */
-  NAO_GEMM_TC = 1     /* BF16 tensor cores on exact 6-bit digit planes of the FP64 operands
-                         (60-bit splitting, FP32-exact partial sums; FP64-level accuracy);
-                         contractions longer than 896 run as chunks summed in FP64.  With
+  NAO_GEMM_TC = 1     /* tensor cores on exact digit planes of the FP64 operands (63-bit
+                         splittings, base 128 in BF16 up to 256 terms, base 32 in E4M3
+                         beyond; FP32-exact partial sums; FP64-level accuracy);
+                         contractions longer than 1232 run as chunks summed in FP64.  With
                          this method the Householder matrix-vector products also run on
-                         exact 8-bit digits (62 bits, int32 dot products on the integer
-                         pipe) up to the order whose digits fit a block (n ~ 3200)        */
+                         exact 8-bit digits (62 bits, FP16 tensor-core products) up to the
+                         order whose column fits the blocks' shared memory (n = 3649);
+                         matrices small enough for it are reduced in one FP64 launch      */
 };
 
 /* Library / context ------------------------------------------------------------------ */

@@ -23,7 +23,9 @@
 //    after the product, one after the next column has been formed.  The dot product of
 //    Procedure 5 needs no third: p^H v = p_raw^H v - 2 Re(y1^H y2) with y1 = W^H v, y2 = V^H v;
 //  * up to 16 blocks share a matrix (tiles of 16 rows dealt out in turn), each keeping its own
-//    rows of the panel's V and W in shared memory where they fit;
+//    rows of the panel's V and W in shared memory where they fit; where a column and its digits (48 n
+//    bytes) do not, the column lies in the digits' space, for one more barrier and pass over v a
+//    column (digits to n = 3649);
 //  * a block pushes its rows of the next column straight into the shared memory of the
 //    others, so that after the barrier the column is local everywhere;
 //  * the panel's own products (V^H v and W^H v, the corrections V y1 + W y2, the next column's
@@ -430,14 +432,17 @@ struct PanelSmem {
   size_t bytes;
 };
 
-__host__ __device__ inline PanelSmem panel_smem(int n, int C, int D, size_t limit) {
+// shared: x lies in the first half of vd (the real part's digits).  The digits are dead once every
+// block has formed its products (B2), which is before the next column is pushed, and v's digits
+// are formed from x through a copy of its real parts in the rings, which are idle then.
+__host__ __device__ inline PanelSmem panel_smem(int n, int C, int D, size_t limit, bool shared) {
   PanelSmem s;
   const int NT = hd_tiles(n);
   s.own = (NT + C - 1) / C;
   const int R = 16 * s.own;
   s.PS = (16 * NT + 63) / 64 * 64 + 16;
   int o = 0;
-  s.x = o, o += 16 * NT;
+  s.x = o, o += shared ? 0 : 16 * NT;
   s.v = o, o += R;
   s.p = o, o += R;
   s.un = o, o += R;
@@ -448,6 +453,7 @@ __host__ __device__ inline PanelSmem panel_smem(int n, int C, int D, size_t limi
   s.ys = o, o += 2 * NB;
   s.slots = o, o += (HP_SLOTS + HP_SLOTS2) * 32;
   s.vd = o, o += 2 * s.PS;
+  if (shared) s.x = s.vd;
   s.cd = o, o += 2 * 2 * HP_PS;
   s.ring = o, o += HP_MMA_WARPS * D * 128;  // (of every warp when the panel's digits come from global memory)
   s.md = o;
@@ -470,7 +476,7 @@ constexpr size_t HP_SMEM_LIMIT = 225 * 1024;  // of 227 KB: the kernel's static 
 //                    M coef (the contraction runs over the panel's columns).
 // Bytes not written yet are digits of finite values that meet zero coefficients or rows that
 // nothing reads.
-template <int S, int D>
+template <int S, int D, bool SHARED>
 __global__ void __launch_bounds__(HP_THREADS, 1)
 hetrd_panel_mma_kernel(int n, const int32_t* __restrict__ size, z64* __restrict__ Abase, int ld, long long strideA,
                        double* __restrict__ dbase, double* __restrict__ ebase, z64* __restrict__ taubase,
@@ -502,7 +508,7 @@ hetrd_panel_mma_kernel(int n, const int32_t* __restrict__ size, z64* __restrict_
     }
     return;
   }
-  const PanelSmem L = panel_smem(n, C, D, HP_SMEM_LIMIT);
+  const PanelSmem L = panel_smem(n, C, D, HP_SMEM_LIMIT, SHARED);
   z64 *x = sm + L.x, *v = sm + L.v, *pown = sm + L.p, *unext = sm + L.un, *wown = sm + L.w, *coefs = sm + L.cf,
       *crow = sm + L.cr, *ypart = sm + L.yp, *ysum = sm + L.ys;
   longlong2* slots = (longlong2*)(sm + L.slots);  // of the MMA warps, then of the others
@@ -638,7 +644,13 @@ hetrd_panel_mma_kernel(int n, const int32_t* __restrict__ size, z64* __restrict_
       }
       const int lt = div_c(r >> 4);
       if (lt * C + rank == r >> 4) ((double*)&v[16 * lt + (r & 15)])[part] = active ? val : 0.0;
-      hp_put(vd + (size_t)part * 8 * PS + r, PS, val, 1);
+      if (SHARED && part == 0) ((double*)(sm + L.ring))[r] = val;  // (x is still being read)
+      else hp_put(vd + (size_t)part * 8 * PS + r, PS, val, 1);
+    }
+    if (SHARED) {
+      __syncthreads();
+#pragma unroll 1
+      for (int r = 16 * ks0 + tid; r < 16 * NT; r += HP_THREADS) hp_put(vd + r, PS, ((const double*)(sm + L.ring))[r], 1);
     }
     if (tid >= HP_THREADS - 128) {  // the next column's coefficients' digits
       const int c = (tid & 127) >> 1, part = tid & 1;
@@ -923,28 +935,39 @@ int smem_optin() {
 
 constexpr int HP_MAX_CLUSTER = 16;  // (beyond 8: the non-portable size)
 
-// Stages of the rings: four, or two where that makes room for the panel's digits or for the
-// vectors of a large matrix; 0: does not fit.
-int panel_stages(int n, int C) {
-  const PanelSmem s4 = panel_smem(n, C, 4, HP_SMEM_LIMIT), s2 = panel_smem(n, C, 2, HP_SMEM_LIMIT);
-  if (s4.md_in_smem) return 4;
-  if (s2.md_in_smem) return 2;
-  return s4.bytes <= HP_SMEM_LIMIT ? 4 : s2.bytes <= HP_SMEM_LIMIT ? 2 : 0;
+// Form of a panel at order n with C blocks a matrix: stages of the rings (four, or two where that makes
+// room for the panel's digits or for the vectors of a large matrix; 0: does not fit), and whether x
+// lies in vd's space, where there is no room for both.
+struct PanelForm {
+  int D;
+  bool shared;
+};
+
+PanelForm panel_form(int n, int C) {
+  const PanelSmem s4 = panel_smem(n, C, 4, HP_SMEM_LIMIT, false), s2 = panel_smem(n, C, 2, HP_SMEM_LIMIT, false);
+  if (s4.md_in_smem) return {4, false};
+  if (s2.md_in_smem) return {2, false};
+  if (s4.bytes <= HP_SMEM_LIMIT) return {4, false};
+  if (s2.bytes <= HP_SMEM_LIMIT) return {2, false};
+  return {panel_smem(n, C, 2, HP_SMEM_LIMIT, true).bytes <= HP_SMEM_LIMIT ? 2 : 0, true};
 }
 
 typedef void (*PanelFn)(int, const int32_t*, z64*, int, long long, double*, double*, z64*, long long, int, const uint4*,
                         const int*, uint4*, z64*, long long);
 
-PanelFn panel_fn(int digits, int D) {
-  if (digits == 6) return D == 4 ? hetrd_panel_mma_kernel<6, 4> : hetrd_panel_mma_kernel<6, 2>;
-  return D == 4 ? hetrd_panel_mma_kernel<HD_S, 4> : hetrd_panel_mma_kernel<HD_S, 2>;
+template <int S>
+PanelFn panel_fn_s(PanelForm f) {
+  if (f.shared) return hetrd_panel_mma_kernel<S, 2, true>;
+  return f.D == 4 ? hetrd_panel_mma_kernel<S, 4, false> : hetrd_panel_mma_kernel<S, 2, false>;
 }
 
-cudaError_t panel_config(PanelFn fn, cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, int n, int nprob, int C, int D,
+PanelFn panel_fn(int digits, PanelForm f) { return digits == 6 ? panel_fn_s<6>(f) : panel_fn_s<HD_S>(f); }
+
+cudaError_t panel_config(PanelFn fn, cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, int n, int nprob, int C, PanelForm f,
                          cudaStream_t st) {
   cfg.gridDim = dim3((unsigned)(nprob * C));
   cfg.blockDim = dim3(HP_THREADS);
-  cfg.dynamicSmemBytes = panel_smem(n, C, D, HP_SMEM_LIMIT).bytes;
+  cfg.dynamicSmemBytes = panel_smem(n, C, f.D, HP_SMEM_LIMIT, f.shared).bytes;
   cfg.stream = st;
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = C;
@@ -961,48 +984,54 @@ cudaError_t panel_config(PanelFn fn, cudaLaunchConfig_t& cfg, cudaLaunchAttribut
 
 bool hetrd_digits_fit(int n, int digits) {
   (void)digits;
-  return panel_stages(n, HP_MAX_CLUSTER) > 0 && (size_t)smem_optin() >= HP_SMEM_LIMIT + 1024;
+  return panel_form(n, HP_MAX_CLUSTER).D > 0 && (size_t)smem_optin() >= HP_SMEM_LIMIT + 1024;
 }
 
 size_t hetrd_panel_bytes(int n, int nprob) {
   const int NT = hd_tiles(n);
-  if (panel_smem(n, 1, 2, HP_SMEM_LIMIT).md_in_smem) return 16;  // (also with more blocks)
+  if (panel_smem(n, 1, 2, HP_SMEM_LIMIT, false).md_in_smem) return 16;  // (also with more blocks)
   return (size_t)(NT + HP_MAX_CLUSTER - 1) * 2 * HP_MDT * 16 * (size_t)nprob;
 }
 
 // Largest cluster size C (16, 8 .. 1; at most one block per 16 rows) for which the nprob
-// clusters of C blocks are all resident at once, as the occupancy calculator reports; more
-// when a matrix's vectors only fit in the shared memory of more blocks.
+// clusters of C blocks are all resident at once, as the occupancy calculator reports.  Where none is:
+// the fewest blocks that a matrix's vectors fit in, beside x unless that takes more than twice as many
+// as in x's space (fewer blocks leave fewer waves; with one or two more or less it is even).
+// Stage `hetrd`, ms, x apart -> in vd's space: n = 2300, 16 problems (C = 7 -> 8) 529 -> 323, 64 problems (7 -> 3)
+// 1471 -> 1174; n = 2500, 16 problems (16 -> 8) 620 -> 417, 64 problems (16 -> 4) 2106 -> 1224; n = 1250, 170
+// problems (2 -> 1) 509 -> 583, which stays apart; n = 3000, 16 problems (FP64 form -> 8) 2131 -> 627.
 int hetrd_mma_cluster_size(int n, int nprob, int num_sms, int digits) {
   const int NT = hd_tiles(n);
-  int fit = 1;
-  while (fit < HP_MAX_CLUSTER && panel_stages(n, fit) == 0) fit = fit < 8 ? fit + 1 : HP_MAX_CLUSTER;
+  const auto next = [](int c) { return c < 8 ? c + 1 : HP_MAX_CLUSTER; };
+  int fit = 1, own = 1;
+  while (fit < HP_MAX_CLUSTER && panel_form(n, fit).D == 0) fit = next(fit);
+  while (own < HP_MAX_CLUSTER && (panel_form(n, own).D == 0 || panel_form(n, own).shared)) own = next(own);
   for (int c = HP_MAX_CLUSTER; c > fit; c = c > 8 ? 8 : c - 1) {
     if (c > NT || (long long)nprob * c > num_sms) continue;
-    const int D = panel_stages(n, c);
-    const PanelFn fn = panel_fn(digits, D);
+    const PanelForm f = panel_form(n, c);
+    const PanelFn fn = panel_fn(digits, f);
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
     int clusters = 0;
-    if (panel_config(fn, cfg, attr, n, nprob, c, D, nullptr) != cudaSuccess ||
+    if (panel_config(fn, cfg, attr, n, nprob, c, f, nullptr) != cudaSuccess ||
         cudaOccupancyMaxActiveClusters(&clusters, fn, &cfg) != cudaSuccess) {
       cudaGetLastError();
       continue;
     }
     if (clusters >= nprob) return c;
   }
-  return fit;
+  return own <= 2 * fit && !panel_form(n, own).shared ? own : fit;
 }
 
 cudaError_t launch_hetrd_panel_mma(int n, int nprob, const int32_t* size, z64* A, int ld, long long strideA, double* d,
                                    double* e, z64* tau, long long strideV, int i0, int C, const void* dig,
                                    const int* erow, int digits, void* md, z64* VWr, long long strideVW, cudaStream_t st) {
-  const int D = panel_stages(n, C);
-  if ((digits != 6 && digits != HD_S) || D == 0) return cudaErrorInvalidValue;
-  const PanelFn fn = panel_fn(digits, D);
+  const PanelForm f = panel_form(n, C);
+  if ((digits != 6 && digits != HD_S) || f.D == 0) return cudaErrorInvalidValue;
+  const PanelFn fn = panel_fn(digits, f);
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
-  const cudaError_t err = panel_config(fn, cfg, attr, n, nprob, C, D, st);
+  const cudaError_t err = panel_config(fn, cfg, attr, n, nprob, C, f, st);
   if (err != cudaSuccess) return err;
   return cudaLaunchKernelEx(&cfg, fn, n, size, A, ld, strideA, d, e, tau, strideV, i0, (const uint4*)dig, erow,
                             (uint4*)md, VWr, strideVW);
