@@ -30,12 +30,12 @@
 //   orthogonalised by kernel 3, one block per cluster, in ascending order (classical
 //   Gram-Schmidt applied twice against the finished members): two vectors with a gap g overlap by at
 //   most ~eps|T|/g, so taking one out of the other changes its residual by overlap x g, of order
-//   eps|T| again.  A member that loses nearly all of its norm (its random start fell into the
-//   others' span) is iterated again from another start with the orthogonalisation inside
-//   the iteration, its solves in one thread.  A chain can span far more than the tight band; a member
-//   is orthogonalised only against the finished members within the band of its own
-//   eigenvalue (the others overlap it by at most eps|T| over the band, which the Newton-Schulz
-//   steps remove).  (Before, one thread walked each cluster of up to 32 members and ran all
+//   eps|T| again over the share of its norm that is left.  A member that loses more than half of its
+//   norm is solved for again, from what is left or (its random start fell into the others' span)
+//   from another start, with the orthogonalisation inside the iteration and the solves in one
+//   thread.  A chain can span far more than the tight band; in one of more than BIG members,
+//   a member is orthogonalised only against the finished ones within the band of its own
+//   eigenvalue (the others overlap it by at most eps|T| over the band).  (Before, one thread walked each cluster of up to 32 members and ran all
 //   solves of larger ones: n = 600, 8 problems with 12 null directions each, 85 -> 18 ms.)
 // * Output: eigenvalues ascending (across blocks), eigenvectors in matching columns,
 //   unit 2-norm, largest component positive.  All loops are bounded.
@@ -59,7 +59,7 @@ constexpr double TIGHT_GS = 1e-11;  // ...and below this, Gram-Schmidt (without 
                                     // them, Gram-Schmidt starts at TIGHT: the big clusters that the
                                     // wider band chains go to MRRR, which needs no serial walk)
 constexpr int NARR = 6;           // scratch arrays per eigenvalue: L, U0inv, U1, U2, PIV, X
-constexpr int BIG = 32;           // tight clusters with more members take kernel 0's vectors when it runs
+constexpr int BIG = 32;           // tight clusters with more members take kernel 0's vectors when it runs, and only their band in kernel 3
 constexpr int NEWTON_MAX = 6;     // Newton steps on an isolated eigenvalue before it is queued
 constexpr int BQ_LANES = 4;       // lanes per queued eigenvalue in the FP64 bisection (multisection), at least
 
@@ -738,8 +738,8 @@ stein_vec_kernel(int n, const int32_t* __restrict__ size, const double* __restri
 // ---------------------------------------------------------------- kernel 3: tight clusters
 // One block per cluster listed by kernel 2: members in ascending order.  Kernel 2's vector is
 // orthogonalised by the block against the finished members (classical Gram-Schmidt, twice); one
-// whose norm falls below CL_KEEP is iterated anew: thread 0 factors T - lambda I and runs the
-// solves (as kernel 2), the block re-orthogonalises each iterate and takes the norms.
+// whose norm falls below CL_DONE is solved for again: thread 0 factors the shifted T - lambda I and
+// runs the solves (as kernel 2), the block re-orthogonalises each iterate and takes the norms.
 __device__ __forceinline__ double block_sum1(double v, double* red) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
 #pragma unroll
@@ -764,7 +764,17 @@ __device__ __forceinline__ double block_max1(double v, double* red) {
 }
 
 constexpr int SC_THREADS = 256;
-constexpr double CL_KEEP = 1e-2;  // (1 - norm^2 is the share of the others: rounding grows by 1 / CL_KEEP at most)
+// What is left of a member's norm after the others are taken out, c, scales its rounding by 1 / c.  From
+// CL_DONE on that is let be; from CL_KEEP on one more solve from what is left takes it away, below three do
+// (from another random start below CL_LEFT).  These solves are shifted by CL_SHIFT eps |T| beyond the
+// member's eigenvalue: within a group of equal eigenvalues T - lambda I amplifies one direction, fixed by
+// rounding, far more than the others, and that may lie among the finished members; the shift is as far
+// from all of them, so that the solve changes nothing within the group.
+// Largest |H v - eps v| / eps |H| over groups of 4, 12, 25 equal eigenvalues (n = 24, 48, 100): one walk of
+// each cluster, every solve orthogonalised, 8, 10, 12; Gram-Schmidt alone from 1e-2 on 179, 477, 1447;
+// solves at the unshifted eigenvalue 8, 302, 78; this 8, 12, 12.  (Stage `stein` of n = 600, 8 problems
+// with 12 null directions each: 17.3 -> 18.3 ms for the solves; the walk took 85.)
+constexpr double CL_DONE = 0.5, CL_KEEP = 1e-2, CL_LEFT = 1e-8, CL_SHIFT = 10.0;
 
 __global__ void __launch_bounds__(SC_THREADS, 1)
 stein_cluster_kernel(int n, const int32_t* __restrict__ size, const double* __restrict__ dbase,
@@ -816,19 +826,16 @@ stein_cluster_kernel(int n, const int32_t* __restrict__ size, const double* __re
     double* __restrict__ U1 = scr + 2 * nn;
     double* __restrict__ U2 = scr + 3 * nn;
     double* __restrict__ PV = scr + 4 * nn;
-    double lamprev = 0.0, ulast = 0.0;
+    double ulast = 0.0;
     bool fail = false;
     const int nv = min(nvec ? nvec[p] : m, nvec_max);
     const int* dn = mdone ? mdone + (size_t)p * n : nullptr;
     for (int q = j; q < jend; ++q) {
       if (rnk[q - j] >= nv) break;  // uniform: ranks ascend with q
-      if (dn && dn[q]) {  // an MRRR vector (kernel 0) is already in Z
-        lamprev = w[q];
-        continue;
-      }
-      if (tid == 0) {  // finished members within the tight band of w[q]: the earlier ones and
-                       // the later MRRR vectors
-        const double tband = tgs * T.onenrm, wq = w[q];
+      if (dn && dn[q]) continue;  // an MRRR vector (kernel 0) is already in Z
+      if (tid == 0) {  // finished members: the earlier ones and the later MRRR vectors, of a big cluster
+                       // those within the tight band of w[q]
+        const double tband = jend - j > BIG ? tgs * T.onenrm : INFINITY, wq = w[q];
         int c = 0;
         for (int t = 0; t < jend - j; ++t)
           if ((t < q - j || (t > q - j && dn && dn[j + t])) && fabs(w[j + t] - wq) < tband) fin[c++] = t;
@@ -866,15 +873,12 @@ stein_cluster_kernel(int n, const int32_t* __restrict__ size, const double* __re
       double a0 = 0.0;
       for (int i = b0 + tid; i < b1; i += nt) a0 = fma(sx[i], sx[i], a0);
       const double kept = block_sum1(a0, red);
-      const bool again = !(kept >= CL_KEEP * CL_KEEP && kept <= 4.0);  // uniform (NaN: again)
-      if (again) {
+      if (!(kept >= CL_DONE * CL_DONE && kept <= 4.0)) {  // uniform (NaN: iterated)
+      const bool fresh = !(kept >= CL_LEFT * CL_LEFT && kept <= 4.0);
+      const int solves = kept >= CL_KEEP * CL_KEEP && !fresh ? 1 : EXTRA + 1;
+      const double shift = CL_SHIFT * eps * T.tnorm;
       if (tid == 0) {  // LU with partial pivoting of T[b0:b1) - lam I (as kernel 2)
-        double lam = w[q];
-        if (q > j) {
-          const double pertol = 10.0 * fabs(eps * lam);
-          if (lam - lamprev < pertol) lam = lamprev + pertol;
-        }
-        lamprev = lam;
+        const double lam = w[q] + shift;
         double al = d[b0] - lam, be = e[b0];
         for (int k = b0; k < b1 - 1; ++k) {
           const double c = e[k];
@@ -913,8 +917,9 @@ stein_cluster_kernel(int n, const int32_t* __restrict__ size, const double* __re
         ulast = al;
         AT(U0i, b1 - 1) = 1.0 / al;
       }
-      for (int i = b0 + tid; i < b1; i += nt)
-        sx[i] = hash_uniform(((unsigned long long)p << 40) ^ ((unsigned long long)q << 20) ^ (unsigned long long)i);
+      if (fresh)  // (not kernel 2's start)
+        for (int i = b0 + tid; i < b1; i += nt)
+          sx[i] = hash_uniform(((unsigned long long)p << 40) ^ ((unsigned long long)q << 20) ^ (unsigned long long)i ^ (1ull << 63));
       __syncthreads();
       int its = 0, nrmchk = 0;
       bool ok = false;
@@ -924,7 +929,7 @@ stein_cluster_kernel(int n, const int32_t* __restrict__ size, const double* __re
         for (int i = b0 + tid; i < b1; i += nt) a1 += fabs(sx[i]);
         const double x1 = block_sum1(a1, red);
         if (tid == 0) {  // scaled right-hand side, forward and back substitution
-          const double scl = (double)bs * T.onenrm * fmax(eps, fabs(ulast)) / fmax(x1, DBL_MIN);
+          const double scl = (double)bs * fmax(T.onenrm * fmax(eps, fabs(ulast)), shift) / fmax(x1, DBL_MIN);
           double r = sx[b0] * scl;
           #pragma unroll 8
           for (int k = b0; k < b1 - 1; ++k) {
@@ -962,13 +967,11 @@ stein_cluster_kernel(int n, const int32_t* __restrict__ size, const double* __re
         if (its > maxits && nrmchk == 0) break;
         if (xinf < sqrt(0.1 / bs)) continue;
         ++nrmchk;
-        if (nrmchk < EXTRA + 1) continue;
+        if (nrmchk < solves) continue;
         ok = true;
         break;
       }
       if (!ok) fail = true;
-      } else {
-        lamprev = w[q];
       }
       // normalise, sign: largest component positive (first of equal magnitude)
       double a2 = 0.0, big = 0.0;
