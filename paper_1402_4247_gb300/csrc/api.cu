@@ -544,7 +544,8 @@ __global__ void ns2_cols_kernel(int nprob, const int* __restrict__ flag, const i
 }
 
 // The second Newton-Schulz step, for the problems the tridiagonal solve flagged (ns2) because
-// a gap in [1e-11, 1e-9) |T|_1 left overlaps up to ~1e-5 that one step reduces only to ~1e-10.
+// a gap in [1e-11, 1e-9) |T|_1, or a big cluster wider than 1e-11 |T|_1, left overlaps up to ~1e-5
+// that one step reduces only to ~1e-10.
 // Tensor-core method: in place, the other problems' columns counted as zero; FP64 CUDA cores:
 // all problems, into the other array.  Returns the array that holds the result.
 double* ns_second(nao_ctx* ctx, int n, int nprob, const int32_t* size, const int32_t* ncols, const int* ns2,

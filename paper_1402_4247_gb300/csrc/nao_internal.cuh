@@ -232,7 +232,8 @@ cudaError_t launch_stein(int n, int nprob, const int32_t* size, const double* d,
                          int mrrr, cudaStream_t st, int* ns2 = nullptr);
 int stein_launches(int n, int nprob, int mrrr);  // kernels of one launch_stein
 // ns2 (nullable, [nprob]): set to 1 for a problem whose vectors need a second Newton-Schulz
-// step (a gap in [1e-11, 1e-9) |T|_1, where inverse iteration leaves overlaps up to ~1e-5)
+// step (a gap in [1e-11, 1e-9) |T|_1, or a cluster of more than 32 wider than 1e-11 |T|_1, where
+// inverse iteration leaves overlaps up to ~1e-5)
 
 // Overlap chain by Cholesky (csrc/chol.cu): the diagonal block of one step (B = 32 or 64 columns
 // from j0; Y: B x B per matrix; fail[p] set where a pivot is not positive), the decision per matrix

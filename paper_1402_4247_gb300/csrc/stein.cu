@@ -25,7 +25,7 @@
 //   overlaps of order eps|T|/gap, which the caller removes with Newton-Schulz steps
 //   Z <- Z (3I - Z^T Z)/2 (each squares them): one step for gaps >= 1e-9 |T|_1 (overlaps <= ~1e-7),
 //   a second one for the problems flagged in ns2[] because a gap lies in [1e-11, 1e-9) |T|_1
-//   (overlaps <= ~1e-5).
+//   or a cluster of more than BIG members is wider than its band (overlaps <= ~1e-5).
 //   The members of a tight cluster (gap < 1e-11 |T|_1; 1e-9 |T|_1 when kernel 0 runs) are then
 //   orthogonalised by kernel 3, one block per cluster, in ascending order (classical
 //   Gram-Schmidt applied twice against the finished members): two vectors with a gap g overlap by at
@@ -584,6 +584,8 @@ stein_vec_kernel(int n, const int32_t* __restrict__ size, const double* __restri
     if (close_hi && !close_lo) {  // the first member lists the cluster for kernel 3
       int jend = j + 2;
       while (jend < b1 && w[jend] - w[jend - 1] < tight) ++jend;
+      // (kernel 3 leaves the members of a big cluster that are a tight band apart to Newton-Schulz)
+      if (ns2 && jend - j > BIG && tight < tight1 && !(w[jend - 1] - w[j] < tight)) ns2[p] = 1;
       const int slot = atomicAdd(&biglist[0], 1);
       if (slot < bigcap) {
         biglist[1 + 3 * slot] = p;
