@@ -581,6 +581,7 @@ stein_vec_kernel(int n, const int32_t* __restrict__ size, const double* __restri
   if (j < m) {
     const int b0 = bst[j], b1 = ben[j];
     const bool close_lo = j > b0 && w[j] - w[j - 1] < tight, close_hi = j + 1 < b1 && w[j + 1] - w[j] < tight;
+    const bool member = close_lo || close_hi;  // of a tight cluster
     if (close_hi && !close_lo) {  // the first member lists the cluster for kernel 3
       int jend = j + 2;
       while (jend < b1 && w[jend] - w[jend - 1] < tight) ++jend;
@@ -710,11 +711,12 @@ stein_vec_kernel(int n, const int32_t* __restrict__ size, const double* __restri
           if (its > maxits && nrmchk == 0) break;
           if (xinf < sqrt(0.1 / bs)) continue;
           ++nrmchk;
-          if (nrmchk < (close_lo || close_hi ? EXTRA : EXTRA_ISOLATED) + 1) continue;
+          if (nrmchk < (member ? EXTRA : EXTRA_ISOLATED) + 1) continue;
           ok = true;
           break;
         }
-        if (!ok) s_fail = 1;
+        // a cluster's member that has not converged is left zero: kernel 3 iterates it and says whether it fails
+        if (!ok && !member) s_fail = 1;
         double nrm2 = 0.0, big = 0.0;
         int jmax = b0;
         for (int i = b0; i < b1; ++i) {
@@ -725,10 +727,10 @@ stein_vec_kernel(int n, const int32_t* __restrict__ size, const double* __restri
             jmax = i;
           }
         }
-        double sc = (nrm2 > 0.0 && nrm2 <= DBL_MAX) ? 1.0 / sqrt(nrm2) : 0.0;
+        double sc = (nrm2 > 0.0 && nrm2 <= DBL_MAX && (ok || !member)) ? 1.0 / sqrt(nrm2) : 0.0;
         if (AT(X, jmax) < 0.0) sc = -sc;
-        for (int i = 0; i < m; ++i) zc[i] = (i >= b0 && i < b1) ? AT(X, i) * sc : 0.0;
-        if (sc == 0.0) zc[b0 + (q - b0) % bs] = 1.0;  // keep a unit vector even on failure
+        for (int i = 0; i < m; ++i) zc[i] = (i >= b0 && i < b1 && sc != 0.0) ? AT(X, i) * sc : 0.0;
+        if (sc == 0.0 && !member) zc[b0 + (q - b0) % bs] = 1.0;  // keep a unit vector even on failure
       } while (false);
 #undef AT
     }
@@ -833,14 +835,14 @@ stein_cluster_kernel(int n, const int32_t* __restrict__ size, const double* __re
     const int nv = min(nvec ? nvec[p] : m, nvec_max);
     const int* dn = mdone ? mdone + (size_t)p * n : nullptr;
     for (int q = j; q < jend; ++q) {
-      if (rnk[q - j] >= nv) break;  // uniform: ranks ascend with q
+      if (rnk[q - j] >= nv) continue;  // (uniform)
       if (dn && dn[q]) continue;  // an MRRR vector (kernel 0) is already in Z
       if (tid == 0) {  // finished members: the earlier ones and the later MRRR vectors, of a big cluster
                        // those within the tight band of w[q]
         const double tband = jend - j > BIG ? tgs * T.onenrm : INFINITY, wq = w[q];
         int c = 0;
         for (int t = 0; t < jend - j; ++t)
-          if ((t < q - j || (t > q - j && dn && dn[j + t])) && fabs(w[j + t] - wq) < tband) fin[c++] = t;
+          if ((t < q - j || (t > q - j && dn && dn[j + t])) && rnk[t] < nv && fabs(w[j + t] - wq) < tband) fin[c++] = t;
         s_nf = c;
       }
       const int sl = q;
