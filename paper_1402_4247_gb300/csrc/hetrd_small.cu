@@ -19,12 +19,15 @@
 //    are formed by one warp and reductions run only in warps that hold rows: with every warp
 //    forming them redundantly a column took 15,000 cycles whatever n.
 // FP64 work per column and block: 12 multiply-adds per element, 6 L^2 / C cycles (L trailing rows).
-// Rule (hetrd_small_cluster): n^2 / C <= 9000 (12000 up to n = 136), where that pass costs less than
-// the panel's longer chain (csrc/hetrd.cu).  Whole reduction, this against panels, us: n = 64, 4
-// problems 422 / 846; n = 100, 150 problems (C = 1) 1599 / 2247; n = 129, 76 problems (C = 2)
-// 1779 / 2653; n = 160, 37 problems (C = 4) 2341 / 3089; n = 211, 24 problems (C = 5) 3270 / 4140; n = 305,
-// 1 problem (C = 16) 4772 / 5595; at the line n = 256, 9 problems (C = 8) 4473 / 4375, n = 360, 1 problem
-// (C = 16) 6786 / 6849.
+// Rule (hetrd_small_cluster): n^2 / C <= 6600, where that pass costs less than the panel's longer chain
+// (csrc/hetrd.cu); up to n = 136, where the blocks are few (C = 1 up to n = 109, C = 2) and their exchange
+// is short, 12000.  Whole reduction with digits and updates, this against panels, us:
+//   C = 1, 150 problems: n = 64 569 / 924, 100 1605 / 1934, 109 1946 / 2034;
+//   C = 2, 76 problems: n = 129 1785 / 2113, 136 2087 / 2281, 150 2752 / 2574;
+//   C = 8, 10 problems: n = 100 718 / 1414, 200 2328 / 3046, 229 3113 / 3548;
+//   C = 16, 1 to 7 problems: n = 64 423 / 792, 200 2094 / 2956, 305 4778 / 5102, 320 5300 / 5366.
+// Clusters over nearly all SMs exchange more slowly and lose up to a tenth near the line: 9 problems
+// (C = 16) n = 200 2761 / 3026, 256 4480 / 3914; 25 problems (C = 6) n = 140 1798 / 2042, 160 2443 / 2303.
 #include <cooperative_groups.h>
 
 #include "nao_internal.cuh"
@@ -296,7 +299,7 @@ int hetrd_small_cluster(int n, int nprob, int num_sms) {
     return 0;
   }
   for (int c = HS_MAX_CLUSTER; c > 0; c = c > 8 ? 8 : c - 1) {
-    if (n * n > c * (n <= 136 ? 12000 : 9000)) return 0;
+    if (n * n > c * (n <= 136 ? 12000 : 6600)) return 0;
     if (c > 1 && (4 * c > n || (long long)nprob * c > num_sms)) continue;
     if (small_smem(n, c).bytes > HS_SMEM_LIMIT) return 0;
     if (c == 1) return 1;
