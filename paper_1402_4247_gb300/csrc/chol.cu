@@ -31,7 +31,7 @@
 // Measured (ms per step; the overlap's chain before -> now, the skipped launches included): n = 64,
 // 4 k-points ~1.3 -> 0.3; n = 305, 27 k-points ~10 -> 2.0; n = 568, 1 k-point ~18 -> 2.5, 64 k-points
 // ~60 -> 8.8; n = 2000, 1 k-point ~140 -> 14.  An overlap that fails pays it on top (n = 600, 8
-// k-points, cut directions: 3.6 of 131).
+// k-points, cut directions: 3.5 of 57 ms).
 #include <cfloat>
 
 #include "nao_internal.cuh"

@@ -42,7 +42,7 @@
 //    taken by all 16 warps from a shared counter, 114 KB: 6.9 ms).
 // A column is now bound by its chain of short phases (~7 us at n = 305), with one block per
 // matrix by the stream of digits (16 B per entry and column: at n = 568, 128 problems, the
-// first columns run at 78 % of the measured HBM rate).
+// first columns run at 4.6 to 4.8 TB/s of DRAM, 69 to 72 % of the measured rate).
 // Measured (stage `hetrd` per step, ms, the FP64 panel's products -> now): n = 305, 27 problems
 // 24.8 -> 4.6; n = 449, 40 problems 39.8 -> 10.6; n = 568, 2 problems 52 -> 9.9; 128 problems
 // 79.3 -> 36.2; n = 2000, 1 problem 458 -> 89.

@@ -234,7 +234,8 @@ __device__ __forceinline__ void oz_pack(uint32_t (&pk)[S][4], int scale0, Q q) {
 // k > j.  Outside it the products are exact zeros, so results do not depend on the range.  An
 // empty range (a later chunk of a long contraction) becomes the first step.
 // Half of H X and X V and a third of the lower triangle of X^H Y are such zeros; measured at
-// n = 568, 128 problems (ms, splits included): H X 10.5 -> 7.1, X^H Y 7.2 -> 6.1, X V 10.6 -> 7.1.
+// n = 568, 128 problems (ms, splits included, ten base-64 planes): H X 10.5 -> 7.1, X^H Y 7.2 -> 6.1, X V
+// 10.6 -> 7.1 (6.0, 5.1 and 6.1 with thirteen e4m3 planes).
 template <int BK>
 __device__ __forceinline__ void oz_krange(const GemmDims& d, int p, int K, int row0, int row1, int col1, int& klo, int& khi) {
   klo = 0, khi = K;
